@@ -17,6 +17,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "device.cuh"
 #include "internal.h"
 
 namespace archead {
@@ -27,7 +28,189 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// One warp per scale group of gr x gc elements of x [rows][cols].
+// Codes of a value v against a scale s > 0 with reciprocal inv = 1 / s: the
+// integer (as a float) clamp(rint(v / s), -qmax, qmax) of the definition
+// above, bit for bit, without its division.  v * inv differs from the
+// rounded quotient by at most 2^-22 of its size, below 5e-5 for the |v / s|
+// <= 1.5 qmax < 200 that a group's own scale leaves (fp16 subnormal scales
+// included), so unless v * inv lies within 1e-4 of a half-integer both round
+// to the same integer; the rest (about 1 value in 5000), and NaNs and
+// infinities, take the division.  Adding 1.5 * 2^23 rounds to an integer,
+// ties to even.
+__device__ __forceinline__ float quant_code(float v, float s, float inv, float qmax) {
+  const float q = v * inv;
+  float r = __fadd_rn(__fadd_rn(q, 12582912.f), -12582912.f);
+  if (!(fabsf(q - r) < 0.4999f)) r = rintf(__fdiv_rn(v, s));
+  return fminf(fmaxf(r, -qmax), qmax);
+}
+
+// Four codes as the bytes of a word.
+__device__ __forceinline__ uint32_t quant_code4(float4 v, float s, float inv, float qmax) {
+  if (!(s > 0.f)) return 0;
+  const int a = (int)quant_code(v.x, s, inv, qmax), b = (int)quant_code(v.y, s, inv, qmax);
+  const int c = (int)quant_code(v.z, s, inv, qmax), d = (int)quant_code(v.w, s, inv, qmax);
+  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+}
+
+__device__ __forceinline__ float abs_max4(float4 v) {
+  return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+}
+
+// Groups of kGc consecutive values of a row (32, 64, 128 or 256): with whole
+// groups per row the matrix is one flat run of groups.  Memory bound (5 bytes
+// a value).  A warp takes 512 values, four 16-byte loads a lane in flight,
+// and keeps them in registers between the group maxima and the codes, so x is
+// read once; the one-warp-per-group kernel below read it twice, 4 bytes a
+// lane, and divided every value.
+template <int kGc>
+__global__ void __launch_bounds__(256) quantize_rows_kernel(const float4 *__restrict__ x, int64_t n4, float qmax,
+                                                            uint32_t *__restrict__ codes,
+                                                            uint16_t *__restrict__ scales) {
+  constexpr int kU = 4;                               // float4 per lane
+  constexpr int kLanes = kGc / 4 < 32 ? kGc / 4 : 32;  // lanes sharing a group
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t w = blockIdx.x * (int64_t)(blockDim.x >> 5) + (threadIdx.x >> 5); w * (32 * kU) < n4; w += warps) {
+    const int64_t base = w * (32 * kU) + lane;
+    float4 v[kU];
+    float mx[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      v[u] = base + 32 * u < n4 ? __ldcs(x + base + 32 * u) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      mx[u] = abs_max4(v[u]);
+#pragma unroll
+      for (int o = kLanes / 2; o > 0; o >>= 1) mx[u] = fmaxf(mx[u], __shfl_xor_sync(0xffffffffu, mx[u], o));
+    }
+    if (kGc == 256) {  // two of the lane's values a group
+#pragma unroll
+      for (int u = 0; u < kU; u += 2) mx[u] = mx[u + 1] = fmaxf(mx[u], mx[u + 1]);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      const int64_t i = base + 32 * u;
+      if (i >= n4) break;
+      const __half s16 = __float2half_rn(__fdiv_rn(mx[u], qmax));
+      const float s = __half2float(s16);
+      if ((i & (kGc / 4 - 1)) == 0) scales[i / (kGc / 4)] = __half_as_ushort(s16);
+      codes[i] = quant_code4(v[u], s, __frcp_rn(s), qmax);
+    }
+  }
+}
+
+// Groups of gr rows of one column (the core factors: gr = all rows; the
+// correction's right factor: gr = g).  A cluster of blocks takes one group
+// of rows of eight adjacent columns (one 32-byte sector of a row), each
+// block a slice of the rows: column maxima over its slice, the maximum over
+// the cluster through distributed shared memory, then the codes.  With all
+// rows of 128 columns in one group, 16 clusters of eight blocks read x at
+// full sectors from 128 SMs, the second time mostly from L2; one warp per
+// column read one value per sector, on 128 warps in all.
+// kVec: cols is a multiple of 8, x 16-byte and codes 8-byte aligned.
+constexpr int kColThreads = 512;
+template <bool kVec>
+__global__ void __launch_bounds__(kColThreads) quantize_columns_kernel(const float *__restrict__ x, int64_t cols,
+                                                                       int64_t gr, float qmax,
+                                                                       int8_t *__restrict__ codes,
+                                                                       uint16_t *__restrict__ scales) {
+  __shared__ float wmax[kColThreads / 32][8];
+  __shared__ float bmax[8];  // this block's maxima, read by the cluster
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint32_t rank, nrank;
+  asm("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(nrank));
+  const int64_t strips = (cols + 7) / 8;
+  const int64_t job = blockIdx.x / nrank;  // (row group, strip)
+  const int64_t c0 = (job % strips) * 8, r0 = (job / strips) * gr;
+  const int nc = (int)(cols - c0 < 8 ? cols - c0 : 8);
+  const float *xs = x + r0 * cols + c0;
+  int8_t *cs = codes + r0 * cols + c0;
+  const int64_t step = (int64_t)nrank * kColThreads;
+  const int64_t first = (int64_t)rank * kColThreads + threadIdx.x;
+  auto load = [&](int64_t r, float (&v)[8]) {
+    if (kVec) {
+      const float4 a = *reinterpret_cast<const float4 *>(xs + r * cols);
+      const float4 b = *reinterpret_cast<const float4 *>(xs + r * cols + 4);
+      v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) v[j] = j < nc ? xs[r * cols + j] : 0.f;
+    }
+  };
+  float mx[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) mx[j] = 0.f;
+  int64_t r = first;
+  for (; r + 3 * step < gr; r += 4 * step) {  // four rows in flight
+    float v[4][8];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) load(r + u * step, v[u]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) mx[j] = fmaxf(mx[j], fabsf(v[u][j]));
+  }
+  for (; r < gr; r += step) {
+    float v[8];
+    load(r, v);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) mx[j] = fmaxf(mx[j], fabsf(v[j]));
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    mx[j] = warp_max(mx[j]);
+    if (lane == j) wmax[warp][j] = mx[j];
+  }
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    float m = 0.f;
+#pragma unroll
+    for (int w = 0; w < kColThreads / 32; ++w) m = fmaxf(m, wmax[w][threadIdx.x]);
+    bmax[threadIdx.x] = m;
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  float s[8], inv[8];
+  {
+    float m = 0.f;  // lane j < 8 of every warp: column j over the cluster's blocks
+    for (uint32_t b = 0; b < nrank; ++b) {
+      uint32_t addr;
+      float v;
+      asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(addr) : "r"(smem_u32(&bmax[lane & 7])), "r"(b));
+      asm volatile("ld.shared::cluster.f32 %0, [%1];\n" : "=f"(v) : "r"(addr) : "memory");
+      m = fmaxf(m, v);
+    }
+    const __half s16 = __float2half_rn(__fdiv_rn(m, qmax));
+    if (rank == 0 && threadIdx.x < nc) scales[(job / strips) * cols + c0 + threadIdx.x] = __half_as_ushort(s16);
+    const float sj = __half2float(s16);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      s[j] = __shfl_sync(0xffffffffu, sj, j);
+      inv[j] = __frcp_rn(s[j]);
+    }
+  }
+  // No block leaves while another may still read its maxima.
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+#pragma unroll 4
+  for (r = first; r < gr; r += step) {
+    float v[8];
+    load(r, v);
+    uint32_t q[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) q[j] = s[j] > 0.f ? (uint32_t)(int)quant_code(v[j], s[j], inv[j], qmax) & 255u : 0u;
+    if (kVec) {
+      *reinterpret_cast<uint2 *>(cs + r * cols) =
+          make_uint2(q[0] | q[1] << 8 | q[2] << 16 | q[3] << 24, q[4] | q[5] << 8 | q[6] << 16 | q[7] << 24);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (j < nc) cs[r * cols + j] = (int8_t)q[j];
+    }
+  }
+}
+
+// One warp per scale group of gr x gc elements of x [rows][cols]: the shapes
+// that the two kernels above do not take.
 __global__ void quantize_symmetric_kernel(const float *__restrict__ x, int64_t rows, int64_t cols, int64_t gr,
                                           int64_t gc, int qmax, int8_t *__restrict__ codes,
                                           uint16_t *__restrict__ scales) {
@@ -95,6 +278,69 @@ __global__ void quantize_residual_sc4_kernel(const float *__restrict__ r, int64_
   }
 }
 
+// The same for g = 32, 64, 128 or 256 and rows of up to 256 kNV float4
+// (cols <= 8192), 16-byte aligned: a block per row, the row held in
+// registers, so r is read once (5 bytes a value in all, which bounds it).
+// Group maxima come from the kLanes lanes holding a group (two halves, for g
+// = 256, meet in shared memory), the row maximum from the warps'; then one
+// thread per group takes its scale code, scale and reciprocal.  The
+// one-warp-per-row kernel read r twice, 4 bytes a lane, and divided every value.
+constexpr int kSc4Threads = 256;
+template <int kNV>
+__global__ void __launch_bounds__(kSc4Threads) quantize_residual_sc4_rows_kernel(
+    const float4 *__restrict__ r, int64_t rows, int cols4, int lg, uint32_t *__restrict__ codes,
+    uint8_t *__restrict__ qcodes, uint16_t *__restrict__ row_scale) {
+  __shared__ float pmax[kSc4Threads * kNV / 8];  // per 32..128-wide piece of the row
+  __shared__ float wmax[kSc4Threads / 32];
+  __shared__ float2 gs[kSc4Threads * kNV / 8];   // (scale, reciprocal) per group
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g4 = 1 << (lg - 2);          // float4 per group
+  const int lanes = g4 < 32 ? g4 : 32;   // lanes sharing a piece
+  const int lp = lg - 2 < 5 ? lg - 2 : 5;  // log2 of the piece's float4 count
+  const int G = cols4 >> (lg - 2);
+  for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
+    float4 v[kNV];
+#pragma unroll
+    for (int u = 0; u < kNV; ++u) {
+      const int i = threadIdx.x + kSc4Threads * u;
+      v[u] = i < cols4 ? __ldcs(r + row * cols4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    float rmax = 0.f;
+#pragma unroll
+    for (int u = 0; u < kNV; ++u) {
+      const int i = threadIdx.x + kSc4Threads * u;
+      float m = abs_max4(v[u]);
+      for (int o = lanes >> 1; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if ((lane & (lanes - 1)) == 0 && i < cols4) pmax[i >> lp] = m;
+      rmax = fmaxf(rmax, m);
+    }
+    rmax = warp_max(rmax);
+    if (lane == 0) wmax[warp] = rmax;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kSc4Threads / 32; ++w) rmax = fmaxf(rmax, wmax[w]);
+    const __half sr16 = __float2half_rn(__fdiv_rn(rmax, 112.f));
+    const float sr = __half2float(sr16);
+    if (threadIdx.x == 0) row_scale[row] = __half_as_ushort(sr16);
+    for (int grp = threadIdx.x; grp < G; grp += kSc4Threads) {
+      const float m = lg == 8 ? fmaxf(pmax[2 * grp], pmax[2 * grp + 1]) : pmax[grp];
+      int q = 0;
+      if (sr > 0.f) q = min(max((int)ceilf(__fdiv_rn(m, 7.f * sr)) - 1, 0), 15);
+      qcodes[row * G + grp] = (uint8_t)q;
+      const float s = sr * (float)(q + 1);
+      gs[grp] = make_float2(s, __frcp_rn(s));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kNV; ++u) {
+      const int i = threadIdx.x + kSc4Threads * u;
+      if (i >= cols4) break;
+      const float2 sc = gs[i >> (lg - 2)];
+      codes[row * cols4 + i] = quant_code4(v[u], sc.x, sc.y, 7.f);
+    }
+  }
+}
+
 // bits 4: two's complement (or unsigned 0..15) nibbles, byte j of a row =
 // columns 2j (low) and 2j+1 (high), a missing last column packed as 0.
 // bits 5: code j of a row in bits 5j..5j+4 of the row's little-endian bit
@@ -120,6 +366,32 @@ __global__ void pack_codes_kernel(const int8_t *__restrict__ codes, int64_t rows
   }
 }
 
+// 4-bit codes of an even number of columns: rows follow one another without
+// padding, so the arrays are flat.  16 codes (one 16-byte load, four in
+// flight) to 8 bytes a thread; a thread per byte with two 64-bit divisions
+// took most of the packing time.
+__global__ void __launch_bounds__(256) pack_nibbles_kernel(const uint4 *__restrict__ codes, int64_t n16,
+                                                           uint2 *__restrict__ packed) {
+  auto pack8 = [](uint32_t a, uint32_t b) {  // 8 codes -> 4 bytes
+    a &= 0x0F0F0F0Fu;
+    b &= 0x0F0F0F0Fu;
+    return __byte_perm(a | a >> 4, b | b >> 4, 0x6420);
+  };
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (; i + 3 * step < n16; i += 4 * step) {
+    uint4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = __ldcs(codes + i + u * step);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) packed[i + u * step] = make_uint2(pack8(v[u].x, v[u].y), pack8(v[u].z, v[u].w));
+  }
+  for (; i < n16; i += step) {
+    const uint4 v = codes[i];
+    packed[i] = make_uint2(pack8(v.x, v.y), pack8(v.z, v.w));
+  }
+}
+
 // out = code * scale for scales over gr x gc groups (fp32; exact).
 __global__ void dequant_symmetric_kernel(const int8_t *__restrict__ codes, const uint16_t *__restrict__ scales,
                                          int64_t rows, int64_t cols, int64_t gr, int64_t gc, float *__restrict__ out) {
@@ -128,6 +400,30 @@ __global__ void dequant_symmetric_kernel(const int8_t *__restrict__ codes, const
     const int64_t r = e / cols, c = e % cols;
     out[e] = (float)codes[e] * __half2float(__ushort_as_half(scales[(r / gr) * ngc + c / gc]));
   }
+}
+
+// The same for groups of 2^lgc >= 4 consecutive values of a row (the matrix
+// is one flat run of groups): four codes to one 16-byte store a thread, four
+// in flight, no divisions.
+__global__ void __launch_bounds__(256) dequant_rows_kernel(const uint32_t *__restrict__ codes,
+                                                           const uint16_t *__restrict__ scales, int64_t n4, int lgc,
+                                                           float4 *__restrict__ out) {
+  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  auto store = [&](int64_t i, uint32_t w, uint16_t s16) {
+    const float s = __half2float(__ushort_as_half(s16));
+    out[i] = make_float4((float)(int8_t)w * s, (float)(int8_t)(w >> 8) * s, (float)(int8_t)(w >> 16) * s,
+                         (float)(int8_t)(w >> 24) * s);
+  };
+  int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (; i + 3 * step < n4; i += 4 * step) {
+    uint32_t w[4];
+    uint16_t s[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) w[u] = codes[i + u * step], s[u] = scales[(i + u * step) >> (lgc - 2)];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) store(i + u * step, w[u], s[u]);
+  }
+  for (; i < n4; i += step) store(i, codes[i], scales[i >> (lgc - 2)]);
 }
 
 // The paper's format: out = code * s_row * (q + 1).
@@ -158,6 +454,45 @@ archead_status fail_cuda(cudaError_t e) {
   return e == cudaErrorMemoryAllocation ? ARCHEAD_ERR_OOM : ARCHEAD_ERR_CUDA;
 }
 
+bool aligned(const void *p, size_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; }
+
+// Blocks for grid-stride kernels: enough for several a multiprocessor, so
+// that a thread's independent loads are in flight on every one of them.
+unsigned stream_grid(int64_t blocks) { return (unsigned)(blocks < 1 ? 1 : blocks < 152 * 32 ? blocks : 152 * 32); }
+
+template <int kGc>
+void launch_quantize_rows(const float *x, int64_t n, int qmax, int8_t *codes, uint16_t *scales, cudaStream_t s) {
+  quantize_rows_kernel<kGc><<<stream_grid((n + 4095) / 4096), 256, 0, s>>>(
+      reinterpret_cast<const float4 *>(x), n / 4, (float)qmax, reinterpret_cast<uint32_t *>(codes), scales);
+}
+
+cudaError_t launch_quantize_columns(const float *x, int64_t rows, int64_t cols, int64_t gr, int qmax, int8_t *codes,
+                                    uint16_t *scales, cudaStream_t s) {
+  const int64_t jobs = (rows / gr) * ((cols + 7) / 8);
+  const int cluster = gr >= 8 * kColThreads ? 8 : 1;  // blocks sharing a group: at least a row a thread each
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(jobs * cluster));
+  cfg.blockDim = dim3(kColThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  const bool vec = cols % 8 == 0 && aligned(x, 16) && aligned(codes, 8);
+  return cudaLaunchKernelEx(&cfg, vec ? quantize_columns_kernel<true> : quantize_columns_kernel<false>, x, cols, gr,
+                            (float)qmax, codes, scales);
+}
+
+template <int kNV>
+void launch_sc4_rows(const float *r, int64_t rows, int64_t cols, int lg, int8_t *codes, uint8_t *qcodes,
+                     uint16_t *row_scale, cudaStream_t s) {
+  quantize_residual_sc4_rows_kernel<kNV><<<stream_grid(rows), kSc4Threads, 0, s>>>(
+      reinterpret_cast<const float4 *>(r), rows, (int)(cols / 4), lg, reinterpret_cast<uint32_t *>(codes), qcodes,
+      row_scale);
+}
+
 int qmax_of(int bits) { return bits == 8 ? 127 : bits == 5 ? 15 : bits == 4 ? 7 : 0; }
 
 }  // namespace
@@ -172,8 +507,24 @@ ARCHEAD_API archead_status archead_quantize_symmetric(const float *x, int64_t ro
   if (rows == 0 || cols == 0) return ARCHEAD_OK;
   if (!x || !codes || !scales) return ARCHEAD_ERR_INVALID_ARG;
   const int64_t ngroups = (rows / group_rows) * (cols / group_cols);
-  quantize_symmetric_kernel<<<grid_for(ngroups * 32), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      x, rows, cols, group_rows, group_cols, qmax_of(bits), codes, scales);
+  const int qmax = qmax_of(bits);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const bool vec = group_rows == 1 && aligned(x, 16) && aligned(codes, 4);
+  if (vec && group_cols == 32) {
+    launch_quantize_rows<32>(x, rows * cols, qmax, codes, scales, s);
+  } else if (vec && group_cols == 64) {
+    launch_quantize_rows<64>(x, rows * cols, qmax, codes, scales, s);
+  } else if (vec && group_cols == 128) {
+    launch_quantize_rows<128>(x, rows * cols, qmax, codes, scales, s);
+  } else if (vec && group_cols == 256) {
+    launch_quantize_rows<256>(x, rows * cols, qmax, codes, scales, s);
+  } else if (group_cols == 1 && group_rows >= kColThreads && ngroups <= (1 << 24)) {
+    cudaError_t e = launch_quantize_columns(x, rows, cols, group_rows, qmax, codes, scales, s);
+    if (e != cudaSuccess) return fail_cuda(e);
+  } else {
+    quantize_symmetric_kernel<<<grid_for(ngroups * 32), 256, 0, s>>>(x, rows, cols, group_rows, group_cols, qmax,
+                                                                     codes, scales);
+  }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? ARCHEAD_OK : fail_cuda(e);
 }
@@ -186,9 +537,19 @@ ARCHEAD_API archead_status archead_quantize_residual_sc4(const float *r, int64_t
   if (!r || !codes || !scale_codes || !row_scale) return ARCHEAD_ERR_INVALID_ARG;
   const int64_t G = cols / group_size;
   if (G > 1024) return ARCHEAD_ERR_UNSUPPORTED;  // per-warp group maxima in shared memory
-  const size_t smem = (size_t)8 * G * sizeof(float);
-  quantize_residual_sc4_kernel<<<grid_for(rows * 32), 256, smem, static_cast<cudaStream_t>(stream)>>>(
-      r, rows, cols, group_size, codes, scale_codes, row_scale);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  const int lg = group_size == 32 ? 5 : group_size == 64 ? 6 : group_size == 128 ? 7 : group_size == 256 ? 8 : 0;
+  const int64_t per = cols / 4;  // float4 a row
+  if (lg && per <= 8 * kSc4Threads && aligned(r, 16) && aligned(codes, 4)) {
+    if (per <= kSc4Threads) launch_sc4_rows<1>(r, rows, cols, lg, codes, scale_codes, row_scale, s);
+    else if (per <= 2 * kSc4Threads) launch_sc4_rows<2>(r, rows, cols, lg, codes, scale_codes, row_scale, s);
+    else if (per <= 4 * kSc4Threads) launch_sc4_rows<4>(r, rows, cols, lg, codes, scale_codes, row_scale, s);
+    else launch_sc4_rows<8>(r, rows, cols, lg, codes, scale_codes, row_scale, s);
+  } else {
+    const size_t smem = (size_t)8 * G * sizeof(float);
+    quantize_residual_sc4_kernel<<<grid_for(rows * 32), 256, smem, s>>>(r, rows, cols, group_size, codes, scale_codes,
+                                                                        row_scale);
+  }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? ARCHEAD_OK : fail_cuda(e);
 }
@@ -199,8 +560,14 @@ ARCHEAD_API archead_status archead_pack_codes(const int8_t *codes, int64_t rows,
   if (rows == 0 || cols == 0) return ARCHEAD_OK;
   if (!codes || !packed) return ARCHEAD_ERR_INVALID_ARG;
   const int64_t row_bytes = bits == 4 ? (cols + 1) / 2 : (5 * cols + 7) / 8;
-  pack_codes_kernel<<<grid_for(rows * row_bytes), 256, 0, static_cast<cudaStream_t>(stream)>>>(codes, rows, cols,
-                                                                                               bits, packed, row_bytes);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (bits == 4 && rows * cols % 16 == 0 && cols % 2 == 0 && aligned(codes, 16) && aligned(packed, 8)) {
+    const int64_t n16 = rows * cols / 16;
+    pack_nibbles_kernel<<<stream_grid((n16 + 1023) / 1024), 256, 0, s>>>(reinterpret_cast<const uint4 *>(codes), n16,
+                                                                         reinterpret_cast<uint2 *>(packed));
+  } else {
+    pack_codes_kernel<<<grid_for(rows * row_bytes), 256, 0, s>>>(codes, rows, cols, bits, packed, row_bytes);
+  }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? ARCHEAD_OK : fail_cuda(e);
 }
@@ -212,8 +579,19 @@ ARCHEAD_API archead_status archead_dequant_symmetric(const int8_t *codes, const 
     return ARCHEAD_ERR_INVALID_ARG;
   if (rows == 0 || cols == 0) return ARCHEAD_OK;
   if (!codes || !scales || !out) return ARCHEAD_ERR_INVALID_ARG;
-  dequant_symmetric_kernel<<<grid_for(rows * cols), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      codes, scales, rows, cols, group_rows, group_cols, out);
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (group_rows == 1 && group_cols >= 4 && (group_cols & (group_cols - 1)) == 0 && aligned(codes, 4) &&
+      aligned(out, 16)) {
+    int lgc = 2;
+    while (((int64_t)1 << lgc) < group_cols) ++lgc;
+    const int64_t n4 = rows * cols / 4;
+    dequant_rows_kernel<<<stream_grid((n4 + 1023) / 1024), 256, 0, s>>>(reinterpret_cast<const uint32_t *>(codes),
+                                                                        scales, n4, lgc,
+                                                                        reinterpret_cast<float4 *>(out));
+  } else {
+    dequant_symmetric_kernel<<<grid_for(rows * cols), 256, 0, s>>>(codes, scales, rows, cols, group_rows, group_cols,
+                                                                   out);
+  }
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? ARCHEAD_OK : fail_cuda(e);
 }

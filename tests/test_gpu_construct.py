@@ -80,6 +80,68 @@ def test_residual_quantiser_of_the_papers_format_bit_exact(g):
     assert np.array_equal(out.cpu().numpy().astype(np.float64), c * np.repeat(sg, g, axis=1))
 
 
+def _edge_values(seed, shape):
+    """Values across many scales, near half-integers of their scale, zero groups and ties of the maximum."""
+    rng = np.random.default_rng(seed)
+    x = rng.standard_normal(shape).astype(np.float32)
+    half = rng.random(shape) < 0.3
+    x[half] = (rng.integers(-7, 7, shape)[half] + 0.5).astype(np.float32) * np.float32(0.25)
+    x *= np.exp2(rng.integers(-30, 12, (shape[0], 1))).astype(np.float32)  # down to fp16 subnormal scales and below
+    x[shape[0] // 2] = 0.0
+    return x
+
+
+def _quantise_at(x, gr, gc, bits, offset):
+    """The quantiser on buffers that start `offset` elements past an allocation."""
+    import torch
+
+    R, C = x.shape
+    xd = torch.empty(R * C + offset, dtype=torch.float32, device="cuda")
+    xd[offset:] = _dev(x).view(-1)
+    codes = torch.zeros(R * C + offset, dtype=torch.int8, device="cuda")
+    scales = torch.zeros((R // gr, C // gc), dtype=torch.int16, device="cuda")
+    view = codes[offset:].view(R, C)
+    archead.archead_quantize_symmetric(xd[offset:].view(R, C), gr, gc, bits, view, scales)
+    return view.cpu().numpy(), scales.cpu().numpy().view(np.uint16)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("shape,groups,bits", [
+    ((3, 32), (1, 32), 4), ((37, 192), (1, 64), 4), ((5, 1664), (1, 128), 8), ((9, 768), (1, 256), 5),  # rows
+    ((511, 3), (511, 1), 8), ((512, 7), (512, 1), 8), ((4095, 16), (4095, 1), 5), ((4096, 16), (4096, 1), 8),
+    ((20011, 13), (20011, 1), 8), ((1200, 24), (600, 1), 4),                                            # columns
+], ids=str)
+def test_quantiser_routes_bit_exact(shape, groups, bits, offset):
+    x = _edge_values(shape[0] + bits, shape)
+    codes, scales = _quantise_at(x, *groups, bits, offset)
+    rq, rs = oc.quantize_symmetric(x, groups[0], groups[1], bits)
+    assert np.array_equal(scales, rs)
+    assert np.array_equal(codes, rq)
+
+
+@pytest.mark.parametrize("cols,g", [(32, 32), (1024, 256), (1056, 32), (2112, 64), (4096, 128), (8192, 256), (8256, 64)])
+def test_sc4_residual_row_widths_bit_exact(cols, g):
+    import torch
+
+    x = _edge_values(cols + g, (11, cols))
+    rc = torch.empty(x.shape, dtype=torch.int8, device="cuda")
+    rq = torch.empty((11, cols // g), dtype=torch.uint8, device="cuda")
+    rs = torch.empty(11, dtype=torch.int16, device="cuda")
+    archead.archead_quantize_residual_sc4(_dev(x), g, rc, rq, rs)
+    c, q, s = oc.quantize_residual_sc4(x, g)
+    assert np.array_equal(rs.cpu().numpy().view(np.uint16), s)
+    assert np.array_equal(rq.cpu().numpy(), q)
+    assert np.array_equal(rc.cpu().numpy(), c)
+
+
+@pytest.mark.parametrize("rows,cols", [(1, 16), (3, 32), (8, 2), (129, 1040), (3, 34)])
+def test_nibble_packer_routes_bit_exact(rows, cols):
+    from paper_2608_02703_gb300 import construct as gc
+
+    c = np.random.default_rng(rows).integers(-8, 8, (rows, cols)).astype(np.int8)
+    assert np.array_equal(gc.pack(_dev(c), 4).cpu().numpy(), oc.pack_int4(c))
+
+
 def test_packers_bit_exact():
     from paper_2608_02703_gb300 import construct as gc
 
