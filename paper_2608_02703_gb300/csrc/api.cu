@@ -221,16 +221,32 @@ archead_status run_prefill(archead_pack *p, const void *x, int64_t M, void *out,
     ce_part_off = c.take((size_t)p->num_tiles * prefill_parts_per_vt() * M * sizeof(float2));
     tlogit_off = c.take((size_t)M * sizeof(float));
   }
+  // Few tokens: the pre-pass that splits d over blocks (the tensor-core one
+  // runs M / 64 blocks per 32 columns, each over the whole of d).
+  const bool split_pre = M <= kPrefillSplitPrepass;
+  size_t partial_off = 0;
+  if (split_pre) {
+    partial_off = c.take(prepass_partial_bytes((int)M, p->lr, p->d));
+    AH_CUDA(ensure_counters(p, prepass_pairs((int)M, p->lr), s));
+  }
   AH_CUDA(ensure_workspace(p, c.off, s));
   PrepassParams pp = prepass_params(p, x, M);
   pp.ts = nullptr;
   pp.T = at<uint16_t>(p->ws, t_off);
-  AH_CUDA(launch_prepass_t(pp, p->lr_t, p->d_pad, s, p));
+  if (split_pre) {
+    pp.partial = at<float>(p->ws, partial_off);
+    pp.counters = p->counters;
+    AH_CUDA(launch_prepass(pp, s, p));
+  } else {
+    AH_CUDA(launch_prepass_t(pp, p->lr_t, p->d_pad, s, p));
+  }
   float2 *ce_part = ce_mode ? at<float2>(p->ws, ce_part_off) : nullptr;
   float *tlogit = ce_mode ? at<float>(p->ws, tlogit_off) : nullptr;
   cudaEvent_t ev = nullptr;
   timer_begin(p, "prefill", s, &ev);
-  cudaError_t e = launch_prefill(p, x, (int)M, pp.T, out, out_fp32, greedy, targets, row0, ce_part, tlogit, s);
+  // The kernel overlaps the pre-pass grid (programmatic dependent launch).
+  const bool pdl = p->lr > 0 && !p->profiling;
+  cudaError_t e = launch_prefill(p, x, (int)M, pp.T, out, out_fp32, greedy, targets, row0, ce_part, tlogit, pdl, s);
   timer_end(p, "prefill", s, ev);
   if (e != cudaSuccess) return cuda_status(e);
   if (ce_mode) {
@@ -252,20 +268,13 @@ archead_status run_forward(archead_pack *p, const void *x, int64_t M, void *out,
   if (path != ARCHEAD_PATH_AUTO && path != ARCHEAD_PATH_DECODE && path != ARCHEAD_PATH_PREFILL)
     return ARCHEAD_ERR_INVALID_ARG;
   AH_CUDA(cudaSetDevice(p->device));
-  // AUTO: one decode launch streams the head once for up to 64 tokens (16,
-  // 32 or 64 per instance); a prefill launch computes full 256-token tiles
-  // and costs about as much as one 64-token decode launch plus a fifth
-  // (Qwen3-8B shape: ~350 us against ~150 us at 32 tokens and ~280 us at 64),
-  // so AUTO decodes up to 64 tokens when that takes at most three launches
-  // (heads too wide for the wide instances' ring run 16-token chunks).
+  // AUTO: up to 16 tokens decode (memory bound, warp-level MMAs); more take
+  // the tensor-core kernel, one pass over the head per 128 tokens.
   // Heads too wide for the decode kernel's shared memory plan (per-group
   // sums of x for 16 tokens, e.g. d = 2^20 at g = 32) take the prefill
   // kernel under AUTO.
-  bool decode = path == ARCHEAD_PATH_DECODE;
-  if (path == ARCHEAD_PATH_AUTO && M <= kDecodeWideTokens && decode_supported(p->d_pad, p->nls_dec, p->g)) {
-    const int tok = decode_variant_tokens(decode_variant(p, (int)M));
-    decode = (M + tok - 1) / tok <= 3;
-  }
+  const bool decode = path == ARCHEAD_PATH_DECODE ||
+                      (path == ARCHEAD_PATH_AUTO && M <= kDecodeMaxTokens && decode_supported(p->d_pad, p->nls_dec, p->g));
   if (decode) return run_decode(p, x, M, out, out_fp32, targets, ce, amax_idx, amax_val, row0, parts3, s);
   return run_prefill(p, x, M, out, out_fp32, targets, ce, amax_idx, amax_val, row0, parts3, s);
 }

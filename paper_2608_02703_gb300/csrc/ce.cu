@@ -6,12 +6,14 @@
 //
 //   ce[m] = max + log(sum) - y[m, t_m].
 //
-// Few tokens: one warp per token; lanes stride over the slices and the
-// partial results are merged by a fixed butterfly.  Many tokens: a block per
-// 32 tokens (lane = token, so the slice reads are coalesced); its 32 warps
-// stride over the slices, eight loads in flight per lane, and are merged in
-// warp order.  Both orders are
-// fixed, so the result is deterministic.
+// A cluster of up to eight blocks takes up to 32 tokens: threads are (slice
+// stride, token) with the token fastest, so the reads are coalesced for any
+// token count (one token: consecutive slices), and the blocks of a cluster
+// split the slices.  Bound by reading the partials (8 bytes per token and
+// slice).  Few tokens were one warp each, a chain of dependent loads: 16 us
+// for one token over the 4748 slices of the Qwen3-8B-shaped head; 512 tokens
+// were 16 blocks.  Threads, warps and blocks are merged in a fixed order, so
+// the result is deterministic.
 #include "device.cuh"
 #include "internal.h"
 
@@ -39,104 +41,134 @@ __device__ __forceinline__ void ce_store(const LsePair &acc, int m, const float 
   }
 }
 
-__global__ void ce_finalize_kernel(const float2 *__restrict__ part, int num_parts, const float *__restrict__ tlogit,
-                                   const int32_t *__restrict__ targets, int64_t row0, int64_t V, int M,
-                                   float *__restrict__ ce, int *err) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= M) return;
-  LsePair acc{-INFINITY, 0.f};
-  for (int i = lane; i < num_parts; i += 32) {
-    const float2 v = part[(int64_t)i * M + warp];
-    acc = lse_merge(acc, LsePair{v.x, v.y});
+// Greedy partials merge by (value, row): the larger value, the lower row on
+// ties, so the result is the first maximum as in argmax.
+struct LseMerge {
+  static __device__ __forceinline__ float2 empty() { return make_float2(-INFINITY, 0.f); }
+  static __device__ __forceinline__ float2 merge(float2 a, float2 b) {
+    const LsePair r = lse_merge(LsePair{a.x, a.y}, LsePair{b.x, b.y});
+    return make_float2(r.m, r.s);
   }
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    LsePair o{__shfl_xor_sync(0xffffffffu, acc.m, off), __shfl_xor_sync(0xffffffffu, acc.s, off)};
-    acc = lse_merge(acc, o);
+};
+struct ArgmaxMerge {
+  static __device__ __forceinline__ float2 empty() { return make_float2(-INFINITY, __int_as_float(0x7fffffff)); }
+  static __device__ __forceinline__ float2 merge(float2 a, float2 b) {
+    return b.x > a.x || (b.x == a.x && __float_as_int(b.y) < __float_as_int(a.y)) ? b : a;
   }
-  if (lane == 0) ce_store(acc, warp, tlogit, targets, row0, V, ce, err);
-}
+};
 
-constexpr int kCeWarps = 32;
+constexpr int kFinThreads = 512;
 
-__global__ void __launch_bounds__(kCeWarps * 32) ce_finalize_wide_kernel(const float2 *__restrict__ part, int num_parts,
-                                                               const float *__restrict__ tlogit,
-                                                               const int32_t *__restrict__ targets, int64_t row0,
-                                                               int64_t V, int M, float *__restrict__ ce, int *err) {
-  __shared__ float2 red[kCeWarps][32];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m = blockIdx.x * 32 + lane;
-  LsePair acc{-INFINITY, 0.f};
+// Merged partial of this block's tokens, valid in threads t < tw of the
+// cluster's first block (token blockIdx / cluster * tw + t).  tw: tokens per
+// cluster, a power of two up to 32.
+template <class Op>
+__device__ __forceinline__ float2 merge_partials(const float2 *__restrict__ part, int num_parts, int M, int tw,
+                                                 uint32_t rank, uint32_t nrank) {
+  __shared__ float2 red[kFinThreads];
+  const int t = threadIdx.x;
+  const int strides = kFinThreads / tw;  // slices read at a time by a block
+  const int m = (int)(blockIdx.x / nrank) * tw + (t & (tw - 1));
+  const int step = strides * (int)nrank;
+  float2 acc = Op::empty();
+  asm volatile("griddepcontrol.wait;\n" ::: "memory");  // the forward's partials
   if (m < M) {
-    int i = warp;
-    for (; i + 7 * kCeWarps < num_parts; i += 8 * kCeWarps) {
+    int i = (int)rank * strides + t / tw;
+    for (; i + 7 * step < num_parts; i += 8 * step) {
       float2 v[8];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) v[u] = part[(int64_t)(i + u * kCeWarps) * M + m];
+      for (int u = 0; u < 8; ++u) v[u] = part[(int64_t)(i + u * step) * M + m];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) acc = lse_merge(acc, LsePair{v[u].x, v[u].y});
+      for (int u = 0; u < 8; ++u) acc = Op::merge(acc, v[u]);
     }
-    for (; i < num_parts; i += kCeWarps) {
-      const float2 v = part[(int64_t)i * M + m];
-      acc = lse_merge(acc, LsePair{v.x, v.y});
-    }
+    for (; i < num_parts; i += step) acc = Op::merge(acc, part[(int64_t)i * M + m]);
   }
-  red[warp][lane] = make_float2(acc.m, acc.s);
-  __syncthreads();
-  if (warp != 0 || m >= M) return;
-  for (int w = 1; w < kCeWarps; ++w) acc = lse_merge(acc, LsePair{red[w][lane].x, red[w][lane].y});
-  ce_store(acc, m, tlogit, targets, row0, V, ce, err);
+  red[t] = acc;
+  for (int h = kFinThreads / 2; h >= tw; h >>= 1) {
+    __syncthreads();
+    if (t < h) red[t] = acc = Op::merge(acc, red[t + h]);
+  }
+  if (nrank > 1) {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    if (rank == 0 && t < tw) {
+      for (uint32_t b = 1; b < nrank; ++b) {
+        uint32_t addr;
+        float2 v;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(addr) : "r"(smem_u32(&red[t])), "r"(b));
+        asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+        acc = Op::merge(acc, v);
+      }
+    }
+    // No block leaves while the first may still read its result.
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+  }
+  return acc;
 }
 
-// Greedy decoding: merge the per-slice (value, row) partials of each token in
-// a fixed order (lanes over slices, then a fixed butterfly); ties keep the
-// lowest row, so the result is the first maximum as in argmax.
-__global__ void argmax_finalize_kernel(const float2 *__restrict__ part, int num_parts, int M,
-                                       int32_t *__restrict__ index, float *__restrict__ value) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (warp >= M) return;
-  float bv = -INFINITY;
-  int bi = 0x7fffffff;
-  for (int i = lane; i < num_parts; i += 32) {
-    const float2 v = part[(int64_t)i * M + warp];
-    const int vi = __float_as_int(v.y);
-    if (v.x > bv || (v.x == bv && vi < bi)) {
-      bv = v.x;
-      bi = vi;
-    }
-  }
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-    const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-    if (ov > bv || (ov == bv && oi < bi)) {
-      bv = ov;
-      bi = oi;
-    }
-  }
-  if (lane == 0) {
-    index[warp] = bi;
-    if (value) value[warp] = bv;
+__device__ __forceinline__ void cluster_rank(uint32_t &rank, uint32_t &nrank) {
+  asm("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
+  asm("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(nrank));
+}
+
+__global__ void __launch_bounds__(kFinThreads) ce_finalize_kernel(const float2 *__restrict__ part, int num_parts,
+                                                                  int tw, const float *__restrict__ tlogit,
+                                                                  const int32_t *__restrict__ targets, int64_t row0,
+                                                                  int64_t V, int M, float *__restrict__ ce, int *err) {
+  uint32_t rank, nrank;
+  cluster_rank(rank, nrank);
+  const float2 acc = merge_partials<LseMerge>(part, num_parts, M, tw, rank, nrank);
+  const int m = (int)(blockIdx.x / nrank) * tw + (int)threadIdx.x;
+  if (rank == 0 && (int)threadIdx.x < tw && m < M) ce_store(LsePair{acc.x, acc.y}, m, tlogit, targets, row0, V, ce, err);
+}
+
+__global__ void __launch_bounds__(kFinThreads) argmax_finalize_kernel(const float2 *__restrict__ part, int num_parts,
+                                                                      int tw, int M, int32_t *__restrict__ index,
+                                                                      float *__restrict__ value) {
+  uint32_t rank, nrank;
+  cluster_rank(rank, nrank);
+  const float2 acc = merge_partials<ArgmaxMerge>(part, num_parts, M, tw, rank, nrank);
+  const int m = (int)(blockIdx.x / nrank) * tw + (int)threadIdx.x;
+  if (rank == 0 && (int)threadIdx.x < tw && m < M) {
+    index[m] = __float_as_int(acc.y);
+    if (value) value[m] = acc.x;
   }
 }
+
+// Grid of a finalize launch: tokens per cluster (32, or all of fewer), and
+// one block per cluster while its threads have at most four slices each,
+// else eight.
+struct FinalizeLaunch {
+  int tw = 1;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2] = {};
+  FinalizeLaunch(int num_parts, int M, cudaStream_t s) {
+    while (tw < M && tw < 32) tw *= 2;
+    const int cluster = num_parts <= 4 * (kFinThreads / tw) ? 1 : 8;
+    cfg.gridDim = dim3((unsigned)(((int64_t)M + tw - 1) / tw * cluster));
+    cfg.blockDim = dim3(kFinThreads);
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cluster;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    // Launched while the forward grid drains; it waits for that grid's end
+    // before it reads.
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
 
 cudaError_t launch_argmax_finalize(const float2 *part, int num_parts, int M, int32_t *index, float *value,
                                    cudaStream_t s) {
-  argmax_finalize_kernel<<<(M + 7) / 8, 256, 0, s>>>(part, num_parts, M, index, value);
-  return cudaGetLastError();
+  FinalizeLaunch l(num_parts, M, s);
+  return cudaLaunchKernelEx(&l.cfg, argmax_finalize_kernel, part, num_parts, l.tw, M, index, value);
 }
 
 static cudaError_t launch_finalize(const float2 *part, int num_parts, const float *tlogit, const int32_t *targets,
                                    int64_t row0, int64_t V, int M, float *out, int *err, cudaStream_t s) {
-  if (M >= 32) {
-    ce_finalize_wide_kernel<<<(M + 31) / 32, kCeWarps * 32, 0, s>>>(part, num_parts, tlogit, targets, row0, V, M, out,
-                                                                    err);
-  } else {
-    ce_finalize_kernel<<<(M + 7) / 8, 256, 0, s>>>(part, num_parts, tlogit, targets, row0, V, M, out, err);
-  }
-  return cudaGetLastError();
+  FinalizeLaunch l(num_parts, M, s);
+  return cudaLaunchKernelEx(&l.cfg, ce_finalize_kernel, part, num_parts, l.tw, tlogit, targets, row0, V, M, out, err);
 }
 
 cudaError_t launch_ce_finalize(const float2 *part, int num_parts, const float *tlogit, const int32_t *targets,

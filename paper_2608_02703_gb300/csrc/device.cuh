@@ -197,14 +197,17 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
 // complete yet may be suspended by the hardware for a system-dependent time
 // (no explicit hint: a 1 ms hint measured 1-3 % slower in the prefill kernel,
 // whose pipeline hand-offs are latency-critical).
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
+__device__ __forceinline__ bool mbar_try_wait_a(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
       "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
+      : "r"(bar), "r"(parity)
       : "memory");
   return ok != 0;
+}
+__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
+  return mbar_try_wait_a(smem_u32(bar), parity);
 }
 
 // Bounded wait: spins until the phase with the given parity completed, the
@@ -240,12 +243,13 @@ __device__ __forceinline__ bool elect_one() {
 // mbar_wait for a whole converged warp: every lane calls it and every lane
 // gets the same answer (the decisions are warp votes), so the code after a
 // wait stays warp-uniform.  Same bound and error reporting as mbar_wait.
-__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, int64_t budget,
-                                               volatile int *abort_flag, int *err) {
-  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+// (mbar_wait_warp_a: by shared-memory address.)
+__device__ __forceinline__ bool mbar_wait_warp_a(uint32_t bar, uint32_t parity, int64_t budget,
+                                                 volatile int *abort_flag, int *err) {
+  if (__all_sync(0xffffffffu, mbar_try_wait_a(bar, parity))) return true;
   const long long t0 = clock64();
   while (true) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__all_sync(0xffffffffu, mbar_try_wait_a(bar, parity))) return true;
     if (__any_sync(0xffffffffu, abort_flag != nullptr && *abort_flag)) return false;
     if (__any_sync(0xffffffffu, clock64() - t0 > budget)) {
       if (elect_one()) {
@@ -255,6 +259,10 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, i
       return false;
     }
   }
+}
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, int64_t budget,
+                                               volatile int *abort_flag, int *err) {
+  return mbar_wait_warp_a(smem_u32(bar), parity, budget, abort_flag, err);
 }
 
 // 2-D tensor copy (TMA) of one box at (c0 = column, c1 = row) into shared

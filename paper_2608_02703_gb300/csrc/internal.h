@@ -52,6 +52,7 @@ constexpr int kLrStepBytes = 2048; // 128 rows x 16 codes
 constexpr int kDecodeMaxTokens = 16;   // tokens per chunk of the rank-r fragments (and of noalloc calls)
 constexpr int kDecodeWideTokens = 64;  // tokens of the widest decode launch
 constexpr int kPrepassKSplit = 256;  // d per pre-pass block
+constexpr int kPrefillSplitPrepass = 128;  // largest M whose prefill takes the split pre-pass
 constexpr int64_t kDefaultWaitBudget = 2000000000LL;  // cycles, about one second
 
 struct DecodeParams {
@@ -192,7 +193,7 @@ bool decode_supported(int d_pad, int nls, int g);
 int decode_variant(const archead_pack *p, int M);
 cudaError_t launch_prefill(const archead_pack *pk, const void *x, int M, const uint16_t *T, void *out, int out_fp32,
                            bool argmax, const int32_t *targets, int row0, float2 *ce_part, float *ce_tlogit,
-                           cudaStream_t s);
+                           bool pdl, cudaStream_t s);
 int prefill_parts_per_vt();
 // Greedy second pass: per token the largest (value, row) over the partials,
 // lowest row on ties.

@@ -1,35 +1,48 @@
-// Tensor-core prefill kernel (large M) of the packed LM-head forward (paper,
-// Section 3.2, Eq. 7; no dense W_hat is formed, the residual is dequantised
-// tile by tile inside the kernel as Appendix B allows).
+// Tensor-core kernel (more than 16 tokens) of the packed LM-head forward
+// (paper, Section 3.2, Eq. 7; no dense W_hat is formed, the residual is
+// dequantised tile by tile inside the kernel as Appendix B allows).
 //
-// Tile: 128 vocabulary rows x 256 tokens.  The vocabulary rows are the MMA's
-// M side (one TMEM lane each), the tokens the N side.  Per 64-wide k step:
-//   - a producer warp loads the x tile (256 tokens x 64, bf16, 128-byte
-//     swizzle) with two 2-D TMA copies and the tile's INT4 code chunk with a
-//     1-D bulk copy;
-//   - four converter warps turn the codes into exact bf16 integers and store
-//     them as the K-major, 128-byte-swizzled A operand in shared memory;
-//   - one thread issues four tcgen05.mma (kind::f16, 128x256x16, fp32
-//     accumulate) into one of two TMEM accumulators; a quantisation group
-//     (g of d) always ends in its own accumulator;
-//   - eight promotion warps read each finished group with tcgen05.ld and add
+// A unit of work is one or two 128-row vocabulary tiles x NT tokens (64 or
+// 128).  The vocabulary rows are the MMA's M side (one TMEM lane each), the
+// tokens the N side.  Per 64-wide k step:
+//   - one producer warp loads the x tile (NT tokens x 64, bf16, 128-byte
+//     swizzle) by TMA into its ring, another the tiles' 4 KB code chunks into
+//     theirs, so codes run ahead of x as far as their ring allows;
+//   - a warpgroup per tile turns the codes into exact bf16 integers and stores
+//     them as the A operand in tensor memory: the code layout is that of
+//     m16n8k16 fragments, which is the register layout of tcgen05.st.16x128b;
+//   - one thread issues four tcgen05.mma (kind::f16, 128 x NT x 16, A from
+//     TMEM, B = x from shared memory, fp32 accumulate) per tile into a ring of
+//     TMEM accumulators.  The two tiles take turns, so each x slot feeds two
+//     tiles and one tile's finished group is drained while the other computes;
+//   - a warpgroup per tile reads each finished block with tcgen05.ld and adds
 //     s[row, group] * partial to fp32 registers (group-wise scales cannot be
 //     folded into exact bf16 operands).
-// The rank-r branches are further k steps: A = int8 codes of A_c (factor 1)
-// or A_w (factor = row scale of A_w), B = the pre-pass's bf16 hi/lo split of
-// x V_c and x B_w^T, read through a second tensor map.
+// The rank-r branches are further k steps: 32 columns of int8 codes of A_c
+// (factor 1) or A_w (factor = row scale of A_w), each 16 of them multiplied
+// with the bf16 hi and lo parts of the pre-pass's t, read through a second
+// tensor map.
 //
 // In the paper's packed format (SC4) a group scale is s_row * (q + 1) with a
 // 4-bit code q.  The converters fold q + 1 into the operand (code * (q + 1)
-// stays an exact bf16 integer, |.| <= 128), so the whole residual is one
-// accumulator block promoted once by s_row: no per-group hand-back.
+// stays an exact bf16 integer, |.| <= 128), and blocks are 512 wide,
+// promoted by s_row.
 //
-// Epilogues: logits (each promotion thread stores one row of its 128 tokens),
+// Why A in tensor memory and two tiles a unit: with A and x in shared memory
+// a 128 x 256 x 16 MMA reads 12 KB in its 128 cycles, the x copy of a k step
+// writes 32 KB and the converters 16 KB, together more than the 128 bytes a
+// cycle shared memory moves; that arrangement ran at 62 % of the measured
+// tensor peak.  Here the MMAs of a k step and tile read 16 KB of x, written
+// once for two tiles, in about 280 cycles.  An MMA of at most 128 tokens takes
+// 69-74 cycles whatever its width, so 17 to 128 tokens cost one pass over the
+// head (measured for the Qwen3-8B shape in the launch rule below).
+//
+// Epilogues: logits (each promotion thread stores one row of its tokens),
 // greedy partials (largest logit and its row per token over each warp's 32
 // rows) and cross-entropy partials (max and sum of exp per token over each
 // warp's 32 rows, plus the target's logit).  The cross-entropy and greedy
 // instances read TMEM in the 16x256b shape, so that a thread holds 4 rows
-// of 32 tokens and most of the reduction over rows is thread-local.
+// of NT / 4 tokens and most of the reduction over rows is thread-local.
 #pragma once
 
 #include <cfloat>
@@ -40,21 +53,37 @@
 
 namespace archead {
 
-constexpr int kPfN = 256;                         // tokens per tile
-constexpr int kPfStages = 4;
-constexpr int kPfABytes = kTileRows * 64 * 2;     // 16 KB
-constexpr int kPfBBytes = kPfN * 64 * 2;          // 32 KB
-constexpr int kPfCodeBytes = 4 * kLrStepBytes;    // 8 KB (4 KB of INT4 or 4 low-rank steps)
-constexpr int kPfStageBytes = kPfABytes + kPfBBytes + kPfCodeBytes;
-constexpr int kPfThreads = 512;
-constexpr int kPfTmemCols = 512;                  // two 256-column accumulators
-constexpr int kPfSmem = 1024 + kPfStages * kPfStageBytes + 256;
+constexpr int kPfThreads = 640;  // producers + MMA, two converter and two promotion warpgroups
+constexpr int kPfTmemCols = 512;
 constexpr float kLog2e = 1.4426950408889634f;  // log2(e)
 constexpr float kLn2 = 0.6931471805599453f;    // ln(2)
 
+// Shared-memory rings and TMEM columns for NT tokens a tile.  A stage is 128
+// of d (or four 16-wide rank-r steps).  TMEM: kNB accumulators of NT columns,
+// then two rings (one a converter warpgroup) of kAS A stages (128 rows x 128
+// k, two halves of 32 columns).
+template <int NT>
+struct PfGeom {
+  static constexpr int kBoxBytes = NT * 64 * 2;  // one TMA box of x: 64 of d
+  static constexpr int kXBytes = 2 * kBoxBytes;
+  static constexpr int kXStages = NT == 128 ? 4 : 5;
+  static constexpr int kScaleOff = 4 * kChunkBytes;  // SC4: up to two byte rows of scale codes a tile
+  static constexpr int kCodeSlot = kScaleOff + 4 * kTileRows;
+  static constexpr int kCodeStages = NT == 128 ? 5 : 7;
+  static constexpr int kNB = NT == 128 ? 3 : 4;
+  static constexpr int kAS = NT == 128 ? 1 : 2;
+  static constexpr int kABase = kNB * NT;
+  static constexpr int kCodeOff = kXStages * kXBytes;
+  static constexpr int kBarOff = kCodeOff + kCodeStages * kCodeSlot;
+  static constexpr int kBars = 3 * kXStages + 2 * kCodeStages + 4 * kAS + 2 * kNB + 1;
+  static constexpr int kSmem = 1024 + kBarOff + kBars * 8 + 16;
+  static_assert(kABase + 2 * kAS * 64 <= kPfTmemCols, "TMEM columns");
+  static_assert(kSmem <= 227 * 1024, "shared memory");
+};
+
 struct PrefillParams {
-  CUtensorMap tmap_x;   // bf16 [M][d], box 64 x 128, 128B swizzle
-  CUtensorMap tmap_t;   // bf16 [M][2*LR], box 64 x 128, 128B swizzle
+  CUtensorMap tmap_x;   // bf16 [M][d], box 64 x NT, 128B swizzle
+  CUtensorMap tmap_t;   // bf16 [M][2*LR], box 64 x NT, 128B swizzle
   const uint8_t *codes;
   const uint16_t *scales;  // fp16 group scales (INT8 format)
   const uint8_t *scodes;   // 4-bit group-scale codes (SC4 format)
@@ -62,8 +91,9 @@ struct PrefillParams {
   const uint8_t *lr_codes;
   const uint16_t *s_a;
   int64_t V;
-  int M, num_vt, num_mt, d_pad, G_pad, g, nls, nls_core, rcp, rrp;
-  int sc4, G_pad2;
+  int M, num_vt, num_mt, tl, d_pad, G_pad, g, nls, nls_core;  // tl: vocabulary tiles per unit (1 or 2)
+  int G_pad2;
+  int blk_log2;  // log2 of a residual block's 16-wide steps (g / 16; SC4: kSc4BlockSteps)
   void *out;
   int out_fp32;
   const int32_t *targets;  // global vocabulary rows
@@ -73,6 +103,10 @@ struct PrefillParams {
   int *err;
   int64_t wait_budget;
 };
+
+// SC4: the residual is promoted every 512 of d.  (Longer blocks lose fp32
+// accuracy in the tensor core's running sum; the promotion costs little.)
+constexpr int kSc4BlockLog2 = 5;
 
 // ------------------------------------------------------------------------
 // tcgen05 / TMA wrappers (inline PTX).
@@ -95,44 +129,58 @@ __device__ __forceinline__ void tc_commit(uint64_t *bar) {
                : "memory");
 }
 
-__device__ __forceinline__ void tc_mma(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
+__device__ __forceinline__ void tc_commit_a(uint32_t bar) {  // shared-memory address of the barrier
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
+}
+
+// D (TMEM) = A (TMEM, 128 x 16) * B^T (shared memory) (+ D).
+__device__ __forceinline__ void tc_mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
+                                          uint32_t accumulate) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 
-// 32 lanes x 32 consecutive 32-bit columns starting at taddr (one value per column per thread).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
-  uint32_t r[32];
+// 16 lanes x 32 columns from registers: a[4j + i] is register i of the
+// m16n8k16 A fragment of 16-wide step j (rows t/4 and t/4 + 8 in the lanes,
+// bf16 pairs along k in the columns).
+__device__ __forceinline__ void tmem_st_frag4(uint32_t taddr, const uint32_t (&a)[16]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
-        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
-        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+      "tcgen05.st.sync.aligned.16x128b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(
+          taddr),
+      "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]), "r"(a[8]), "r"(a[9]),
+      "r"(a[10]), "r"(a[11]), "r"(a[12]), "r"(a[13]), "r"(a[14]), "r"(a[15])
+      : "memory");
 }
 
-// 16 lanes x 32 columns starting at taddr (lane field = first lane) in the
-// 16x256b shape, 4 repetitions of 8 columns: in repetition c thread t holds
-// v[4c + j] = (lane t/4 + 8 (j >> 1), column 8c + 2 (t % 4) + (j & 1)).
-__device__ __forceinline__ void tmem_ld16x256b_x4(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+// Loads of 16 registers that tmem_wait_ld completes.  kQuad false: 32 lanes x
+// 16 columns, one value per column (32x32b).  kQuad true: 16 lanes x 32
+// columns in the 16x256b shape: in repetition c thread t holds v[4c + j] =
+// (lane t/4 + 8 (j >> 1), column 8c + 2 (t % 4) + (j & 1)).
+template <bool kQuad>
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  if constexpr (kQuad)
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+  else
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr));
+}
+// The registers pass through the wait, so nothing reads them before it.
+__device__ __forceinline__ void tmem_wait_ld(uint32_t (&r)[16]) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
 }
 
 // 2^x by the special-function unit (ex2.approx, flushes denormal results).
@@ -178,21 +226,10 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int m, int n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-// Byte offset of bf16 element (row, k) in a 128-row x 64 K-major tile with the
-// 128-byte swizzle: 16-byte chunk k/8 of row r is stored at chunk (k/8) ^ (r%8).
-__device__ __forceinline__ uint32_t sw128_off(int row, int k) {
-  return (uint32_t)(row * 128 + ((((k >> 3) ^ (row & 7)) & 7) << 4) + (k & 7) * 2);
+// Prefetch of a contiguous range into L2 (16-byte aligned, size a multiple of 16).
+__device__ __forceinline__ void bulk_prefetch_l2(const void *src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;\n" ::"l"(src), "r"(bytes) : "memory");
 }
-
-// ------------------------------------------------------------------------
-// Promotion blocks of a tile: residual groups, then the core and the
-// correction branches of the extended rank axis.
-// ------------------------------------------------------------------------
-struct BlockPlan {
-  int nres, res_sub;       // residual blocks (groups; one for SC4), 16-wide sub-steps per block
-  int core_sub, corr_sub;  // sub-steps of the core (2*RCP/16) and correction (2*RRP/16) blocks
-  __device__ int nblocks() const { return nres + (core_sub > 0) + (corr_sub > 0); }
-};
 
 // bf16x2 fused multiply-add a * b + c (round to nearest even).
 __device__ __forceinline__ uint32_t bf16x2_fma(uint32_t a, uint32_t b, uint32_t c) {
@@ -201,46 +238,214 @@ __device__ __forceinline__ uint32_t bf16x2_fma(uint32_t a, uint32_t b, uint32_t 
   return d;
 }
 
-// For a 4-bit scale code q: bf16x2 (q+1, q+1) and (-136 (q+1), -136 (q+1)),
-// so that fma(136 + code, m, -136 m) = code * (q + 1) exactly.
-__device__ __forceinline__ void sc4_mult(uint32_t byte, int sh, uint32_t &m2, uint32_t &nb2) {
-  const float m = (float)(((byte >> sh) & 15u) + 1u);
-  m2 = pack_bf16x2(m, m);
-  nb2 = pack_bf16x2(-kInt4Bias * m, -kInt4Bias * m);
+// For a 4-bit scale code q: bf16x2 m = (q+1, q+1) and nb = (-136 (q+1), ...),
+// so that fma(136 + code, m, nb) = code * (q + 1) exactly.  Every step is
+// exact in bf16: 128 + q from the bits, minus 127; 136 (q+1) = 8 * 17 (q+1)
+// has at most 8 significant bits.
+struct Sc4Mult {
+  uint32_t m, nb;
+  __device__ __forceinline__ void set(uint32_t byte, int sh) {
+    const uint32_t b = 0x43004300u + ((byte >> sh) & 15u) * 0x00010001u;
+    m = bf16x2_sub(b, 0x42FE42FEu);  // 127
+    asm("mul.rn.bf16x2 %0, %1, %2;\n" : "=r"(nb) : "r"(m), "r"(0xC308C308u));  // -136
+  }
+};
+
+template <int N>
+struct Int {
+  static constexpr int value = N;
+};
+
+// Position of a ring of N slots: slot and phase parity, advanced in order.
+template <int N>
+struct RingPos {
+  int s = 0;
+  uint32_t ph = 0;
+  __device__ __forceinline__ void next(int by = 1) {
+    s += by;
+    const bool wrap = s >= N;
+    s = wrap ? s - N : s;
+    ph ^= wrap;
+  }
+  __device__ __forceinline__ RingPos ahead(int by) const {
+    RingPos r = *this;
+    r.next(by);
+    return r;
+  }
+};
+
+// After a failed wait: lets the copies a producer has issued land before the
+// block exits (`issued` of them over a ring of n slots; a whole warp calls it).
+__device__ __forceinline__ void drain_copies(uint64_t *full, int n, int issued, int64_t budget, int *err) {
+  for (int k = issued > n ? issued - n : 0; k < issued; ++k)
+    mbar_wait_warp(&full[k % n], (uint32_t)(k / n) & 1, budget, nullptr, err);
 }
 
-// kMode 0: logits, 1: cross-entropy partials, 2: greedy (largest logit, row)
-// partials; kSC4: the paper's packed format (group-scale codes times row scales).
-template <int kMode, bool kSC4>
+// Per-token reductions over a warp's 32 rows of 64 token columns (half HH of
+// the tile's NT), accumulators in the quad layout: acc[(NT/2) h + 4 kk + j] =
+// row 8 (2h + (j >> 1)) + lane / 4, token column 8 kk + 2 (lane % 4) + (j & 1).
+// So a thread holds rows ru + 8 kr (kr = 0..3, ru = lane / 4) of 16 columns
+// col(k) = 8 (k >> 1) + 2 cq + (k & 1), row kr at acc[i0(k) + {0, 2, NT/2,
+// NT/2 + 2}[kr]].  A butterfly over lane bits 4, 3, 2 halves the column set
+// per step: lane (ru, cq) ends with columns 8 ru + 2 cq + j, j = 0, 1.
+template <int NT, int HH>
+__device__ __forceinline__ constexpr int quad_i0(int k) {
+  return 4 * (8 * HH + (k >> 1)) + (k & 1);
+}
+
+// Greedy partials: the largest logit of each token and its row (lowest on ties).
+template <int NT, int HH>
+__device__ __forceinline__ void quad_argmax(const PrefillParams &p, const float (&acc)[NT], int64_t rbase, int64_t part,
+                                            int m0, int lane) {
+  const int ru = lane >> 2, cq = lane & 3;
+  const int valid = rbase + 32 > p.V ? (int)(p.V - rbase) : 32;  // rows of the warp inside V
+  float bv[16];
+  int bi[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int i0 = quad_i0<NT, HH>(k);
+    float v = ru < valid ? acc[i0] : -INFINITY;
+    int ix = ru;
+    if (ru + 8 < valid && acc[i0 + 2] > v) v = acc[i0 + 2], ix = ru + 8;
+    if (ru + 16 < valid && acc[i0 + NT / 2] > v) v = acc[i0 + NT / 2], ix = ru + 16;
+    if (ru + 24 < valid && acc[i0 + NT / 2 + 2] > v) v = acc[i0 + NT / 2 + 2], ix = ru + 24;
+    bv[k] = v;
+    bi[k] = ix;
+  }
+#pragma unroll
+  for (int n = 16, o = 16; n > 2; n >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < n / 2; ++j) {
+      const float kv = up ? bv[j + n / 2] : bv[j];
+      const int ki = up ? bi[j + n / 2] : bi[j];
+      const float gv = up ? bv[j] : bv[j + n / 2];
+      const int gi = up ? bi[j] : bi[j + n / 2];
+      const float rv = __shfl_xor_sync(0xffffffffu, gv, o);
+      const int ri = __shfl_xor_sync(0xffffffffu, gi, o);
+      const bool take = rv > kv || (rv == kv && ri < ki);
+      bv[j] = take ? rv : kv;
+      bi[j] = take ? ri : ki;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int m = m0 + 64 * HH + 8 * ru + 2 * cq + j;
+    if (m < p.M) p.ce_part[part * p.M + m] = make_float2(bv[j], __int_as_float((int)rbase + bi[j]));
+  }
+}
+
+// Cross-entropy partials: (max, sum of exp(y - max)) of each token, and the
+// target's logit.  The accumulators are in units of ln 2.
+template <int NT, int HH>
+__device__ __forceinline__ void quad_ce(const PrefillParams &p, float (&acc)[NT], int64_t rbase, int64_t part, int m0,
+                                        int lane) {
+  const int ru = lane >> 2, cq = lane & 3;
+  m0 += 64 * HH;
+  // Target logits first: a token whose target is one of this warp's 32 rows
+  // takes its value from the thread holding it (rare, so the slow path is a
+  // warp-uniform branch).  Lane (ru, cq) reads the targets of the columns it
+  // ends with.
+  int tg[2];
+  bool hit = false;
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int m = m0 + 8 * ru + 2 * cq + j;
+    const int64_t t64 = m < p.M ? (int64_t)p.targets[m] - p.row0 - rbase : -1;  // row within the warp's 32
+    tg[j] = t64 >= 0 && t64 < 32 ? (int)t64 : -1;
+    hit |= tg[j] >= 0;
+  }
+  if (__any_sync(0xffffffffu, hit)) {
+#pragma unroll
+    for (int col = 0; col < 64; ++col) {
+      const int owner = 4 * (col >> 3) + ((col >> 1) & 3);  // lane that read this column's target
+      const int r = __shfl_sync(0xffffffffu, tg[col & 1], owner);
+      if (r >= 0) {  // warp-uniform
+        const int i0 = 4 * (8 * HH + (col >> 3)) + (col & 1);
+        const float mine =
+            r & 16 ? (r & 8 ? acc[i0 + NT / 2 + 2] : acc[i0 + NT / 2]) : (r & 8 ? acc[i0 + 2] : acc[i0]);
+        const float v = __shfl_sync(0xffffffffu, mine, 4 * (r & 7) + ((col >> 1) & 3));
+        if (lane == owner) p.ce_tlogit[m0 + col] = v * kLn2;
+      }
+    }
+  }
+  // Rows past V (last tile only) enter as -FLT_MAX: weight 0 against any
+  // logit, and a finite (max, count) when the warp holds no real row.
+  if (rbase + 32 > p.V) {
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+      const int i0 = quad_i0<NT, HH>(k);
+      if (rbase + ru >= p.V) acc[i0] = -FLT_MAX;
+      if (rbase + ru + 8 >= p.V) acc[i0 + 2] = -FLT_MAX;
+      if (rbase + ru + 16 >= p.V) acc[i0 + NT / 2] = -FLT_MAX;
+      if (rbase + ru + 24 >= p.V) acc[i0 + NT / 2 + 2] = -FLT_MAX;
+    }
+  }
+  float mx[16], sm[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int i0 = quad_i0<NT, HH>(k);
+    const float v0 = acc[i0], v1 = acc[i0 + 2], v2 = acc[i0 + NT / 2], v3 = acc[i0 + NT / 2 + 2];
+    const float mk = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3));
+    mx[k] = mk;
+    sm[k] = (ex2_approx(v0 - mk) + ex2_approx(v1 - mk)) + (ex2_approx(v2 - mk) + ex2_approx(v3 - mk));
+  }
+#pragma unroll
+  for (int n = 16, o = 16; n > 2; n >>= 1, o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < n / 2; ++j) {
+      const float km = up ? mx[j + n / 2] : mx[j], ks = up ? sm[j + n / 2] : sm[j];
+      const float gm = up ? mx[j] : mx[j + n / 2], gs = up ? sm[j] : sm[j + n / 2];
+      const float rm = __shfl_xor_sync(0xffffffffu, gm, o), rs = __shfl_xor_sync(0xffffffffu, gs, o);
+      lse2_merge(km, ks, rm, rs, mx[j], sm[j]);
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const int m = m0 + 8 * ru + 2 * cq + j;
+    if (m < p.M) p.ce_part[part * p.M + m] = make_float2(mx[j] * kLn2, sm[j]);
+  }
+}
+
+// NT: tokens per tile; kMode 0: logits, 1: cross-entropy partials, 2: greedy
+// (largest logit, row) partials; kSC4: the paper's packed format (group-scale
+// codes times row scales).
+template <int NT, int kMode, bool kSC4>
 __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_constant__ PrefillParams p) {
+  using G = PfGeom<NT>;
+  constexpr int kNB = G::kNB, kAS = G::kAS, kXS = G::kXStages;
   extern __shared__ uint8_t pf_smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t *full = reinterpret_cast<uint64_t *>(smem + kPfStages * kPfStageBytes);
-  uint64_t *a_full = full + kPfStages;
-  uint64_t *empty = a_full + kPfStages;
-  uint64_t *acc_full = empty + kPfStages;
-  uint64_t *acc_empty = acc_full + 2;
-  uint64_t *drain = acc_empty + 2;
+  // ready[t][x slot]: tile t's A stage is converted and, for t = 0, x has
+  // landed (tile 1's MMAs of a stage follow tile 0's).
+  uint64_t *ready = reinterpret_cast<uint64_t *>(smem + G::kBarOff);
+  uint64_t *x_empty = ready + 2 * kXS;
+  uint64_t *c_full = x_empty + kXS;
+  uint64_t *c_empty = c_full + G::kCodeStages;
+  uint64_t *a_empty = c_empty + G::kCodeStages;  // [2][kAS][half]
+  uint64_t *acc_full = a_empty + 4 * kAS;
+  uint64_t *acc_empty = acc_full + kNB;
+  uint64_t *drain = acc_empty + kNB;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int KC = p.d_pad / 64;                 // residual k steps
-  const int KE = (2 * (p.rcp + p.rrp)) / 64;   // extended (rank) k steps
+  const int KC = p.d_pad / 128;      // residual stages
+  const int KE = (p.nls + 3) / 4;    // rank-r stages of four 16-wide steps (the last: two or four)
   const int KS = KC + KE;
-  const int num_tiles = p.num_vt * p.num_mt;
-  BlockPlan bp{kSC4 ? 1 : p.G_pad, kSC4 ? p.d_pad / 16 : p.g / 16, 2 * p.rcp / 16, 2 * p.rrp / 16};
+  const int num_units = (p.num_vt + p.tl - 1) / p.tl * p.num_mt;
+  // Promotion blocks of a tile: residual blocks, then the core and the
+  // correction branches.
+  const int nres = ((KC * 8 - 1) >> p.blk_log2) + 1;
+  const bool has_core = p.nls_core > 0, has_corr = p.nls > p.nls_core;
+  const int nb = nres + has_core + has_corr;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kPfStages; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&a_full[i], 4);
-      mbar_init(&empty[i], 1);
-    }
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&acc_full[i], 1);
-      mbar_init(&acc_empty[i], 8);
-    }
+    for (int i = 0; i < kXS; ++i) mbar_init(&ready[i], 5), mbar_init(&ready[kXS + i], 4), mbar_init(&x_empty[i], 1);
+    for (int i = 0; i < G::kCodeStages; ++i) mbar_init(&c_full[i], 1), mbar_init(&c_empty[i], 8);
+    for (int i = 0; i < 4 * kAS; ++i) mbar_init(&a_empty[i], 1);
+    for (int i = 0; i < kNB; ++i) mbar_init(&acc_full[i], 1), mbar_init(&acc_empty[i], 4);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -252,401 +457,472 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
   const uint32_t tmem_base = *tmem_slot;
   bool mma_leader = false;  // the lane of warp 1 that issues the MMAs
 
-  // Registers are rebalanced between warpgroups (launch: 512 x 128): the
-  // converters keep 88, the producer/MMA warpgroup 88 (logits) or 56 (cross
-  // entropy, greedy), the two promotion warpgroups get the rest, 168 or 184
-  // (128 fp32 accumulators per thread; the 4-row epilogues need more): 4*32*(88 + 88) + 8*32*168 = 4*32*(56 + 88) + 8*32*184 = 65536.
-  // Each role's code follows its own setmaxnreg so that the compiler
-  // allocates within that budget; these splits compile without spills.
+  // Registers are rebalanced between warpgroups (launch: 640 x 96).  128
+  // accumulators a promotion thread leave 160 for those warpgroups, 56 for
+  // the converters, 48 for producers and MMA: 128 * 48 + 256 * 56 + 256 * 160
+  // = 640 * 96; with 64 accumulators 128, 64 and 56.  Each role's code follows
+  // its own setmaxnreg so that the compiler allocates within that budget.
   if (warp < 4) {
-    if constexpr (kMode != 0)
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;\n" ::: "memory");
+    if constexpr (NT == 128)
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 48;\n" ::: "memory");
     else
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 88;\n" ::: "memory");
-  if (warp == 0) {
-    // ------------------------------ producer ------------------------------
-    // The whole warp runs the loop (uniform waits); one elected lane issues.
-    {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;\n" ::: "memory");
+    if (warp == 0) {
+      // ------------------------------ x producer ------------------------------
+      // The whole warp runs the loop (uniform waits); one elected lane issues.
       const bool leader = elect_one();
-      int s = 0;
-      uint32_t ph = 0;
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-        const int vt = t / p.num_mt, mt = t % p.num_mt;
-        const int m0 = mt * kPfN;
+      RingPos<kXS> r;
+      int issued = 0;
+      for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
+        const int m0 = (u % p.num_mt) * NT;
         for (int e = 0; e < KS; ++e) {
-          if (!mbar_wait_warp(&empty[s], ph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
-          uint8_t *st = smem + s * kPfStageBytes;
-          uint8_t *bdst = st + kPfABytes;
-          uint8_t *cdst = bdst + kPfBBytes;
-          if (!leader) {
-          } else if (e < KC) {
-            mbar_arrive_expect_tx(&full[s], kPfBBytes + kChunkBytes + (kSC4 ? kTileRows : 0));
-            tma_load_2d(bdst, &p.tmap_x, e * 64, m0, &full[s]);
-            tma_load_2d(bdst + kPfBBytes / 2, &p.tmap_x, e * 64, m0 + 128, &full[s]);
-            bulk_g2s(cdst, p.codes + ((int64_t)vt * KC + e) * kChunkBytes, kChunkBytes, &full[s]);
-            if constexpr (kSC4)  // the byte row of scale codes holding this k step's groups
-              bulk_g2s(cdst + kChunkBytes, p.scodes + ((int64_t)vt * p.G_pad2 + ((e * 64) >> (__ffs(p.g) - 1) >> 1)) * kTileRows,
-                       kTileRows, &full[s]);
-          } else {
-            const int xe = e - KC;
-            mbar_arrive_expect_tx(&full[s], kPfBBytes + 4 * kLrStepBytes);
-            tma_load_2d(bdst, &p.tmap_t, xe * 64, m0, &full[s]);
-            tma_load_2d(bdst + kPfBBytes / 2, &p.tmap_t, xe * 64, m0 + 128, &full[s]);
-            for (int q = 0; q < 4; ++q) {
-              const int kk = xe * 64 + q * 16;  // column of the extended operand
-              int ls;
-              if (kk < 2 * p.rcp) ls = (kk % p.rcp) / 16;
-              else ls = p.nls_core + ((kk - 2 * p.rcp) % p.rrp) / 16;
-              bulk_g2s(cdst + q * kLrStepBytes, p.lr_codes + ((int64_t)vt * p.nls + ls) * kLrStepBytes, kLrStepBytes,
-                       &full[s]);
+          if (!mbar_wait_warp(&x_empty[r.s], r.ph ^ 1, p.wait_budget, abort_flag, p.err)) {
+            drain_copies(ready, kXS, issued, p.wait_budget, p.err);
+            goto done;
+          }
+          if (e == KC && issued < KS) asm volatile("griddepcontrol.wait;\n" ::: "memory");  // t is the pre-pass grid's
+          if (leader) {
+            uint8_t *dst = smem + r.s * G::kXBytes;
+            if (e < KC) {
+              mbar_arrive_expect_tx(&ready[r.s], G::kXBytes);
+              tma_load_2d(dst, &p.tmap_x, e * 128, m0, &ready[r.s]);
+              tma_load_2d(dst + G::kBoxBytes, &p.tmap_x, e * 128 + 64, m0, &ready[r.s]);
+            } else {
+              const bool two = 4 * (e - KC) + 2 < p.nls;
+              mbar_arrive_expect_tx(&ready[r.s], two ? G::kXBytes : G::kBoxBytes);
+              tma_load_2d(dst, &p.tmap_t, (e - KC) * 128, m0, &ready[r.s]);
+              if (two) tma_load_2d(dst + G::kBoxBytes, &p.tmap_t, (e - KC) * 128 + 64, m0, &ready[r.s]);
             }
           }
-          if (++s == kPfStages) s = 0, ph ^= 1;
+          ++issued;
+          r.next();
           __syncwarp();
         }
       }
-    }
-  } else if (warp == 1) {
-    // ------------------------------ MMA issuer ------------------------------
-    // As for the producer: the warp runs the loop, one elected lane issues.
-    // Keeping the loop warp-uniform (votes on every wait, elect.sync for the
-    // issuing lane) is what lets the MMAs issue back to back.
-    {
+    } else if (warp == 2) {
+      // ------------------------------ code producer ------------------------------
+      const bool leader = elect_one();
+      RingPos<G::kCodeStages> r;
+      int issued = 0;
+      const int lg = __ffs(p.g) - 1;
+      const uint32_t scale_bytes = (uint32_t)p.G_pad * kTileRows * 2;
+      for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
+        const int vt0 = u / p.num_mt * p.tl;
+        const int ntile = min(p.tl, p.num_vt - vt0);
+        if (!kSC4 && leader) {
+          // The group scales are read by the promotion warps from global
+          // memory: bring this block's first and then each next unit's to L2.
+          if (u == (int)blockIdx.x) bulk_prefetch_l2(p.scales + (int64_t)vt0 * p.G_pad * kTileRows, scale_bytes * ntile);
+          const int un = u + (int)gridDim.x;
+          if (un < num_units) {
+            const int vn = un / p.num_mt * p.tl;
+            if (vn != vt0)
+              bulk_prefetch_l2(p.scales + (int64_t)vn * p.G_pad * kTileRows, scale_bytes * min(p.tl, p.num_vt - vn));
+          }
+        }
+        for (int e = 0; e < KS; ++e) {
+          if (!mbar_wait_warp(&c_empty[r.s], r.ph ^ 1, p.wait_budget, abort_flag, p.err)) {
+            drain_copies(c_full, G::kCodeStages, issued, p.wait_budget, p.err);
+            goto done;
+          }
+          if (leader) {
+            uint8_t *dst = smem + G::kCodeOff + r.s * G::kCodeSlot;
+            if (e < KC) {
+              // SC4: the byte rows of scale codes holding this stage's groups.
+              const uint32_t sc = kSC4 ? (lg == 5 ? 2 * kTileRows : kTileRows) : 0;
+              mbar_arrive_expect_tx(&c_full[r.s], (uint32_t)ntile * (2 * kChunkBytes + sc));
+              for (int t = 0; t < ntile; ++t) {
+                const int64_t vt = vt0 + t;
+                bulk_g2s(dst + t * 2 * kChunkBytes, p.codes + (vt * KC + e) * 2 * kChunkBytes, 2 * kChunkBytes,
+                         &c_full[r.s]);
+                if (kSC4)
+                  bulk_g2s(dst + G::kScaleOff + t * 2 * kTileRows,
+                           p.scodes + (vt * p.G_pad2 + ((e * 128) >> lg >> 1)) * kTileRows, sc, &c_full[r.s]);
+              }
+            } else {
+              const uint32_t bytes = min(4, p.nls - 4 * (e - KC)) * kLrStepBytes;
+              mbar_arrive_expect_tx(&c_full[r.s], (uint32_t)ntile * bytes);
+              for (int t = 0; t < ntile; ++t)
+                bulk_g2s(dst + t * 2 * kChunkBytes,
+                         p.lr_codes + ((int64_t)(vt0 + t) * p.nls + 4 * (e - KC)) * kLrStepBytes, bytes, &c_full[r.s]);
+            }
+          }
+          ++issued;
+          r.next();
+          __syncwarp();
+        }
+      }
+    } else if (warp == 1) {
+      // ------------------------------ MMA issuer ------------------------------
+      // As for the producers: the warp runs the loop, one elected lane issues.
+      //
+      // The tiles of a unit take turns of at most one stage of a block (one
+      // rank-r step, hi and lo), so that block starts alternate between the
+      // tiles: accumulator i of the ring is the unit's block (i - base) /
+      // ntile of tile (i - base) % ntile.
+      //
+      // This loop's own instructions bound the kernel unless they are few (one
+      // wait per stage and tile): x arrives on the converters' barrier, and
+      // the converters pass a finished stage on to the x producer.
       const bool leader = elect_one();
       mma_leader = leader;
-      constexpr uint32_t idesc = idesc_bf16(128, kPfN);
-      const uint64_t desc0 = smem_desc_sw128(smem_u32(smem));
-      constexpr uint32_t kStageDesc = kPfStageBytes >> 4;  // descriptor address step of one stage
-      constexpr uint32_t kBDesc = kPfABytes >> 4;           // A -> B within a stage
-      int s = 0;
-      uint32_t ph = 0;
-      int bcount = 0;  // accumulator blocks started so far
-      for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-        int blk = 0, in_blk = 0;
-        int blk_len = bp.nres > 0 ? bp.res_sub : (bp.core_sub > 0 ? bp.core_sub : bp.corr_sub);
-        for (int e = 0; e < KS; ++e) {
-          // The converters arrive on a_full only after the stage's TMA bytes landed.
-          if (!mbar_wait_warp(&a_full[s], ph, p.wait_budget, abort_flag, p.err)) goto done;
-          tc_fence_after();
-          const uint64_t ad = desc0 + (uint64_t)(s * kStageDesc);
-          const uint64_t bd = ad + kBDesc;
+      constexpr uint32_t idesc = idesc_bf16(128, NT);
+      const uint64_t xdesc = smem_desc_sw128(smem_u32(smem));
+      const uint32_t ready_a = smem_u32(ready), a_empty_a = smem_u32(a_empty), acc_full_a = smem_u32(acc_full),
+                     acc_empty_a = smem_u32(acc_empty);
+      constexpr uint32_t kBox = G::kBoxBytes >> 4;  // descriptor step to the second box of a stage
+      RingPos<kXS> xr;
+      RingPos<kAS> ar0, ar1;  // A stages consumed from the converter rings
+      RingPos<kNB> accr;      // next accumulator to start
+
+      auto wait = [&](uint32_t bar, uint32_t ph) { return mbar_wait_warp_a(bar, ph, p.wait_budget, abort_flag, p.err); };
+      // Starts the next accumulator once it is drained: its columns in d, its barrier in f.
+      auto acc_start = [&](uint32_t &d, uint32_t &f) {
+        if (!wait(acc_empty_a + 8 * accr.s, accr.ph ^ 1)) return false;
+        d = tmem_base + accr.s * NT;
+        f = acc_full_a + 8 * accr.s;
+        accr.next();
+        return true;
+      };
+      auto ready_wait = [&](int t) { return wait(ready_a + 8 * (t * kXS + xr.s), xr.ph); };
+      // N MMAs from 16-wide step q0 of a residual stage of ring r; first: the
+      // block starts here; f != 0: it ends here.  A half is released after its last step.
+      auto steps = [&](auto n, int q0, int r, const RingPos<kAS> &ar, uint32_t d, bool first, uint32_t f) {
+        constexpr int N = decltype(n)::value;
+        tc_fence_after();
+        const uint32_t a = tmem_base + G::kABase + (r * kAS + ar.s) * 64 + 8 * q0;
+        const uint32_t ae = a_empty_a + 16 * (r * kAS + ar.s);
+        const uint64_t b = xdesc + (uint32_t)(xr.s * (G::kXBytes >> 4)) + (q0 >> 2) * kBox + 2 * (q0 & 3);
+        if (leader) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int buf = bcount & 1;
-            if (in_blk == 0) {
-              if (!mbar_wait_warp(&acc_empty[buf], ((bcount >> 1) & 1) ^ 1, p.wait_budget, abort_flag, p.err))
-                goto done;
-              tc_fence_after();
+          for (int q = 0; q < N; ++q) {  // +2 in the descriptor: 32 bytes in 16-byte units
+            tc_mma_ts(d, a + 8 * q, b + (q >> 2) * kBox + 2 * (q & 3), idesc, q > 0 || !first);
+            if (N >= 4 && (q & 3) == 3) tc_commit_a(ae + 8 * ((q0 + q) >> 2));
+          }
+          if (N == 2 && (q0 & 2)) tc_commit_a(ae + 8 * (q0 >> 2));
+          if (f) tc_commit_a(f);
+        }
+        __syncwarp();
+      };
+
+      for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
+        const int ntile = min(p.tl, p.num_vt - u / p.num_mt * p.tl);
+        uint32_t d0 = 0, d1 = 0, f0 = 0, f1 = 0;
+        if (p.blk_log2 >= 3) {  // blocks of whole stages
+          const int per = 1 << (p.blk_log2 - 3);
+          int left = 0;  // stages to go in the block
+          for (int e = 0; e < KC; ++e) {
+            const bool first = left == 0;
+            if (first) left = per;
+            --left;
+            const bool last = left == 0 || e + 1 == KC;
+            if (first && !acc_start(d0, f0)) goto done;
+            if (!ready_wait(0)) goto done;
+            if (ntile == 2) {
+              steps(Int<8>{}, 0, 0, ar0, d0, first, last ? f0 : 0);
+              if (first && !acc_start(d1, f1)) goto done;
+              if (!ready_wait(1)) goto done;
+              steps(Int<8>{}, 0, 1, ar1, d1, first, last ? f1 : 0);
+              ar0.next();
+              ar1.next();
+            } else if (e & 1) {
+              steps(Int<8>{}, 0, 1, ar1, d0, first, last ? f0 : 0);
+              ar1.next();
+            } else {
+              steps(Int<8>{}, 0, 0, ar0, d0, first, last ? f0 : 0);
+              ar0.next();
             }
-            // +2 per 16-wide k step: 32 bytes in the descriptor's 16-byte address units.
-            if (leader) tc_mma(tmem_base + buf * kPfN, ad + 2 * q, bd + 2 * q, idesc, in_blk > 0);
-            if (++in_blk == blk_len) {
-              if (leader) tc_commit(&acc_full[buf]);
-              ++bcount;
-              ++blk;
-              in_blk = 0;
-              blk_len = blk < bp.nres ? bp.res_sub : (blk == bp.nres && bp.core_sub > 0 ? bp.core_sub : bp.corr_sub);
+            xr.next();
+          }
+        } else {  // groups of 64 (two blocks a stage) or 32 (four)
+          const int nq = p.blk_log2 == 2 ? 4 : 2;
+          for (int e = 0; e < KC; ++e) {
+            for (int q0 = 0; q0 < 8; q0 += nq) {
+              for (int t = 0; t < ntile; ++t) {
+                uint32_t d, f;
+                if (!acc_start(d, f)) goto done;
+                if (q0 == 0 && !ready_wait(t)) goto done;
+                const int r = ntile == 2 ? t : (e & 1);
+                const RingPos<kAS> ar = r ? ar1 : ar0;
+                if (nq == 4)
+                  steps(Int<4>{}, q0, r, ar, d, true, f);
+                else
+                  steps(Int<2>{}, q0, r, ar, d, true, f);
+              }
+            }
+            if (ntile == 2 || !(e & 1)) ar0.next();
+            if (ntile == 2 || (e & 1)) ar1.next();
+            xr.next();
+          }
+        }
+        // Rank-r columns: step l of a stage is one branch's 16 columns (A
+        // columns 8 l), hi and lo 16 columns of t each.
+        for (int e = KC; e < KS; ++e) {
+          const int n = min(4, p.nls - 4 * (e - KC));
+          for (int l = 0; l < n; ++l) {
+            const int ls = 4 * (e - KC) + l;
+            const bool first = ls == 0 || ls == p.nls_core;
+            const bool last = ls == p.nls_core - 1 || ls == p.nls - 1;
+            for (int t = 0; t < ntile; ++t) {
+              if (first) {
+                uint32_t d, f;
+                if (!acc_start(d, f)) goto done;
+                if (t) d1 = d, f1 = f;
+                else d0 = d, f0 = f;
+              }
+              if (l == 0 && !ready_wait(t)) goto done;
+              tc_fence_after();
+              const int r = ntile == 2 ? t : (e & 1);
+              const uint32_t slot = r * kAS + (r ? ar1.s : ar0.s);
+              const uint32_t a = tmem_base + G::kABase + slot * 64 + 8 * l;
+              const uint64_t b = xdesc + (uint32_t)(xr.s * (G::kXBytes >> 4)) + (l >> 1) * kBox + 4 * (l & 1);
+              const uint32_t d = t ? d1 : d0;
+              if (leader) {
+                tc_mma_ts(d, a, b, idesc, !first);
+                tc_mma_ts(d, a, b + 2, idesc, 1);
+                if (l == n - 1) tc_commit_a(a_empty_a + 16 * slot), tc_commit_a(a_empty_a + 16 * slot + 8);
+                if (last) tc_commit_a(t ? f1 : f0);
+              }
+              __syncwarp();
             }
           }
-          if (leader) tc_commit(&empty[s]);
-          if (++s == kPfStages) s = 0, ph ^= 1;
-          __syncwarp();
+          if (ntile == 2 || !(e & 1)) ar0.next();
+          if (ntile == 2 || (e & 1)) ar1.next();
+          xr.next();
         }
       }
     }
-  }
-  } else if (warp < 8) {
+  } else if (warp < 12) {
     // ------------------------------ converters ------------------------------
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 88;\n" ::: "memory");
-    const int cw = warp - 4;
-    const int gq = lane >> 2, cq = lane & 3;
+    // Warpgroup cg converts tile cg of a unit of two tiles, and every other
+    // stage of a unit of one.
+    if constexpr (NT == 128)
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;\n" ::: "memory");
+    else
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 64;\n" ::: "memory");
+    const int cg = (warp - 4) >> 2, cw = warp & 3;
     const int lg = __ffs(p.g) - 1;  // log2 g
-    int s = 0;
-    uint32_t ph = 0;
-    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(cw * 32) << 16) + G::kABase + cg * kAS * 64;
+    RingPos<G::kCodeStages> r;
+    RingPos<kXS> xr;
+    RingPos<kAS> ar;
+    // x slots of the last kAS stages this warpgroup converted, newest first
+    // (-1: not its to release): when an A stage is free again, the MMAs that
+    // read it and its x slot are done.  The unit's last tile releases x.
+    int held[kAS];
+#pragma unroll
+    for (int i = 0; i < kAS; ++i) held[i] = -1;
+    for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
+      const int ntile = min(p.tl, p.num_vt - u / p.num_mt * p.tl);
+      const int tile = ntile == 2 ? cg : 0;
       for (int e = 0; e < KS; ++e) {
-        if (!mbar_wait_warp(&full[s], ph, p.wait_budget, abort_flag, p.err)) goto done;
-        uint8_t *a_tile = smem + s * kPfStageBytes;
-        const uint8_t *codes = a_tile + kPfABytes + kPfBBytes;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int mi = cw * 2 + h;
+        if (!mbar_wait_warp(&c_full[r.s], r.ph, p.wait_budget, abort_flag, p.err)) goto done;
+        if (ntile == 2 || (e & 1) == cg) {
+          const uint8_t *slot = smem + G::kCodeOff + r.s * G::kCodeSlot;
+          const uint8_t *codes = slot + tile * 2 * kChunkBytes + (cw * 64 + lane) * 16;
+          uint64_t *ae = &a_empty[2 * (cg * kAS + ar.s)];
+          const uint32_t acol = lane_addr + ar.s * 64;
           if (e < KC) {
-            const uint4 w4 = *reinterpret_cast<const uint4 *>(codes + (mi * 32 + lane) * 16);
-            const uint32_t ws[4] = {w4.x, w4.y, w4.z, w4.w};
-            // SC4: scale-code bytes of rows gq and gq + 8; the multipliers q + 1
-            // are set for each 32-wide half of the k step (the halves' groups
-            // differ only when g = 32).
-            uint32_t b_lo = 0, b_hi = 0, m_lo = 0, nb_lo = 0, m_hi = 0, nb_hi = 0;
+            // The warp's codes of the stage first (m-tiles 2 cw and 2 cw + 1 of
+            // two 64-wide halves), then the slot is free; one m-tile's
+            // conversion overlaps the store of the one before.
+            uint4 w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = *reinterpret_cast<const uint4 *>(codes + (i >> 1) * kChunkBytes + (i & 1) * 512);
+            uint32_t q[kSC4 ? 4 : 1];  // SC4: scale-code bytes of rows lane/4 + 8 i
+            uint32_t q1[kSC4 ? 4 : 1];  // and of the second half where g = 32
             if constexpr (kSC4) {
-              b_lo = codes[kChunkBytes + mi * 16 + gq];
-              b_hi = codes[kChunkBytes + mi * 16 + gq + 8];
-            }
+              const uint8_t *sb = slot + G::kScaleOff + tile * 2 * kTileRows + cw * 32 + (lane >> 2);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              uint32_t a[4];
-              if constexpr (kSC4) {
-                if (j % 2 == 0) {
-                  const int sh = 4 * (((e * 64 + 16 * j) >> lg) & 1);  // nibble of the half's group
-                  sc4_mult(b_lo, sh, m_lo, nb_lo);
-                  sc4_mult(b_hi, sh, m_hi, nb_hi);
+              for (int i = 0; i < 4; ++i) q[i] = sb[8 * i];
+              if (lg == 5) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) q1[i] = sb[kTileRows + 8 * i];
+              }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&c_empty[r.s]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int hf = i >> 1, h = i & 1;
+              uint32_t ah[16];
+              const uint32_t ws[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+              Sc4Mult lo, hi;  // SC4: multipliers q + 1 of the half's group (two groups where g = 32)
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                uint32_t a[4];
+                if constexpr (kSC4) {
+                  if (j == 0 || (j == 2 && lg == 5)) {
+                    const int sh = 4 * (((e * 128 + hf * 64 + 16 * j) >> lg) & 1);
+                    const bool second = hf == 1 && lg == 5;
+                    lo.set(second ? q1[2 * h] : q[2 * h], sh);
+                    hi.set(second ? q1[2 * h + 1] : q[2 * h + 1], sh);
+                  }
+                  unpack_int4x8_biased(ws[j], a);
+                  a[0] = bf16x2_fma(a[0], lo.m, lo.nb);
+                  a[1] = bf16x2_fma(a[1], hi.m, hi.nb);
+                  a[2] = bf16x2_fma(a[2], lo.m, lo.nb);
+                  a[3] = bf16x2_fma(a[3], hi.m, hi.nb);
+                } else {
+                  unpack_int4x8(ws[j], a);
                 }
-                unpack_int4x8_biased(ws[j], a);
-                a[0] = bf16x2_fma(a[0], m_lo, nb_lo);
-                a[1] = bf16x2_fma(a[1], m_hi, nb_hi);
-                a[2] = bf16x2_fma(a[2], m_lo, nb_lo);
-                a[3] = bf16x2_fma(a[3], m_hi, nb_hi);
-              } else {
-                unpack_int4x8(ws[j], a);
-              }
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int row = mi * 16 + gq + 8 * (i & 1);
-                const int k = j * 16 + 2 * cq + 8 * (i >> 1);
-                *reinterpret_cast<uint32_t *>(a_tile + sw128_off(row, k)) = a[i];
+                for (int k = 0; k < 4; ++k) ah[4 * j + k] = a[k];
               }
+              if (h == 0) {
+                if (!mbar_wait_warp(ae + hf, ar.ph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
+                tc_fence_after();
+              }
+              tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16) + 32 * hf, ah);
             }
-          } else {
+          } else {  // four rank-r steps: the first half's 32 columns
+            const uint8_t *lc = slot + tile * 2 * kChunkBytes + (cw * 64 + lane) * 8;
+            const int n = p.nls - 4 * (e - KC);
+            uint2 w[8];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const uint2 w2 = *reinterpret_cast<const uint2 *>(codes + q * kLrStepBytes + (mi * 32 + lane) * 8);
-              uint32_t a[4];
-              unpack_int8x8(w2.x, w2.y, a);
+            for (int i = 0; i < 8; ++i)
+              w[i] = i < 4 || n > 2 ? *reinterpret_cast<const uint2 *>(lc + (i >> 1) * kLrStepBytes + (i & 1) * 256)
+                                    : make_uint2(0x80808080u, 0x80808080u);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&c_empty[r.s]);
+            if (!mbar_wait_warp(ae + 1, ar.ph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;  // after the first half's
+            tc_fence_after();
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                const int row = mi * 16 + gq + 8 * (i & 1);
-                const int k = q * 16 + 2 * cq + 8 * (i >> 1);
-                *reinterpret_cast<uint32_t *>(a_tile + sw128_off(row, k)) = a[i];
+            for (int h = 0; h < 2; ++h) {
+              uint32_t ah[16];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                uint32_t a[4];
+                unpack_int8x8(w[2 * j + h].x, w[2 * j + h].y, a);
+#pragma unroll
+                for (int k = 0; k < 4; ++k) ah[4 * j + k] = a[k];
               }
+              tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16), ah);
             }
           }
+          asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) {
+            mbar_arrive(&ready[tile * kXS + xr.s]);
+            if (cw == 0 && held[kAS - 1] >= 0) mbar_arrive(&x_empty[held[kAS - 1]]);
+          }
+          ar.next();
+#pragma unroll
+          for (int i = kAS - 1; i > 0; --i) held[i] = held[i - 1];
+          held[0] = tile == ntile - 1 ? xr.s : -1;
+        } else {
+          if (lane == 0) mbar_arrive(&c_empty[r.s]);
         }
-        fence_proxy_async_smem();  // make the generic-proxy stores visible to the tensor core
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&a_full[s]);
-        if (++s == kPfStages) s = 0, ph ^= 1;
+        r.next();
+        xr.next();
       }
     }
   } else {
     // ------------------------------ promotion + epilogue ------------------------------
-    if constexpr (kMode != 0)
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 184;\n" ::: "memory");
+    if constexpr (NT == 128)
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 160;\n" ::: "memory");
     else
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 168;\n" ::: "memory");
-    const int pw = warp - 8;
-    const int lg = pw & 3;            // TMEM lane group (rows 32*lg .. 32*lg+31)
-    const int ch = pw >> 2;           // column half (tokens 128*ch .. 128*ch+127)
-    const int r_in_tile = lg * 32 + lane;
-    // Cross entropy and greedy read TMEM in the 16x256b shape (4 rows x 32
+      asm volatile("setmaxnreg.inc.sync.aligned.u32 128;\n" ::: "memory");
+    const int tile = (warp - 12) >> 2;  // tile of the unit
+    const int lg = warp & 3;            // TMEM lane group (rows 32*lg .. 32*lg+31)
+    // Cross entropy and greedy read TMEM in the 16x256b shape (4 rows x NT/4
     // tokens per thread; cross entropy accumulates in base 2, its factors
-    // times log2 e); logits read 32x32b (one row x 128 tokens per thread).
+    // times log2 e); logits read 32x32b (one row x NT tokens per thread).
     constexpr bool kQuad = kMode != 0;
-    int bcount = 0;
-    for (int t = blockIdx.x; t < num_tiles; t += gridDim.x) {
-      const int vt = t / p.num_mt, mt = t % p.num_mt;
-      const int m0 = mt * kPfN + ch * 128;
-      const int64_t row = (int64_t)vt * kTileRows + r_in_tile;
-      float acc[128];
+    constexpr int kF = kQuad ? 4 : 1;  // rows per thread
+    const int rt0 = lg * 32 + (kQuad ? lane >> 2 : lane);
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(lg * 32) << 16);
+    RingPos<kNB> base;  // the unit's first accumulator
+    for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
+      const int vt0 = u / p.num_mt * p.tl;
+      const int ntile = min(p.tl, p.num_vt - vt0);
+      RingPos<kNB> accr = base.ahead(tile);
+      {
+        const int end = base.s + nb * ntile;
+        base.s = end % kNB;
+        base.ph ^= (end / kNB) & 1;
+      }
+      if (tile >= ntile) continue;
+      const int64_t vt = vt0 + tile;
+      const int m0 = (u % p.num_mt) * NT;
+      float acc[NT];
 #pragma unroll
-      for (int i = 0; i < 128; ++i) acc[i] = 0.f;
-      const int nb = bp.nblocks();
+      for (int i = 0; i < NT; ++i) acc[i] = 0.f;
+      // Promotion factors of a block's rows (rt0, or rt0 + 8k), fp16 bits, loaded a block ahead.
+      uint16_t fn[kF];
+      const uint16_t *fsrc = (kSC4 ? p.s_row + vt * kTileRows : p.scales + vt * p.G_pad * kTileRows) + rt0;
+#pragma unroll
+      for (int k = 0; k < kF; ++k) fn[k] = fsrc[8 * k];
       for (int b = 0; b < nb; ++b) {
-        // Promotion factor of block b for the thread's row(s) of the tile.
-        float f[kQuad ? 4 : 1];
-        if constexpr (kQuad) {
-          // Rows lane / 4 + 8k of the warp's 32: one base pointer, offsets 8k.
-          const int rt0 = lg * 32 + (lane >> 2);
-          const uint16_t *fs = nullptr;
-          if (b < bp.nres)
-            fs = kSC4 ? p.s_row + (int64_t)vt * kTileRows + rt0
-                      : p.scales + ((int64_t)vt * p.G_pad + b) * kTileRows + rt0;
-          else if (!(b == bp.nres && bp.core_sub > 0)) fs = p.s_a + (int64_t)vt * kTileRows + rt0;
+        float f[kF];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            f[k] = fs ? fp16_bits_to_f32(fs[8 * k]) : 1.f;
-            if (kMode == 1) f[k] *= kLog2e;
+        for (int k = 0; k < kF; ++k) f[k] = fp16_bits_to_f32(fn[k]) * (kMode == 1 ? kLog2e : 1.f);
+        if (b + 1 < nres) {
+          if (!kSC4) {
+            fsrc += kTileRows;
+#pragma unroll
+            for (int k = 0; k < kF; ++k) fn[k] = fsrc[8 * k];
           }
-        } else {
-          if (b < bp.nres)
-            f[0] = kSC4 ? fp16_bits_to_f32(p.s_row[row])
-                        : fp16_bits_to_f32(p.scales[((int64_t)vt * p.G_pad + b) * kTileRows + r_in_tile]);
-          else if (b == bp.nres && bp.core_sub > 0) f[0] = 1.f;
-          else f[0] = fp16_bits_to_f32(p.s_a[row]);
+        } else if (b + 1 == nres && has_core) {
+#pragma unroll
+          for (int k = 0; k < kF; ++k) fn[k] = 0x3C00;  // 1
+        } else if (has_corr) {
+#pragma unroll
+          for (int k = 0; k < kF; ++k) fn[k] = p.s_a[vt * kTileRows + rt0 + 8 * k];
         }
-        const int buf = bcount & 1;
-        if (!mbar_wait_warp(&acc_full[buf], (bcount >> 1) & 1, p.wait_budget, abort_flag, p.err)) goto done;
+        if (!mbar_wait_warp(&acc_full[accr.s], accr.ph, p.wait_budget, abort_flag, p.err)) goto done;
         tc_fence_after();
-        const uint32_t taddr = tmem_base + ((uint32_t)(lg * 32) << 16) + buf * kPfN + ch * 128;
-        if constexpr (kQuad) {
-          // acc[64h + 4kk + j] = row 8 (2h + (j >> 1)) + lane / 4 of the warp's
-          // 32, token column 8kk + 2 (lane % 4) + (j & 1), kk = 0..15.
+        const uint32_t taddr = lane_addr + accr.s * NT;
+        // Chunks of 16 registers, the next one loading while one is added.
+        constexpr int kChunks = NT / 16;
+        auto chunk_addr = [&](int c) {  // quad: rows 16 (c / (NT/32)), columns 32 (c % (NT/32))
+          return kQuad ? taddr + ((uint32_t)(16 * (c / (NT / 32))) << 16) + 32 * (c % (NT / 32)) : taddr + 16 * c;
+        };
+        uint32_t v[2][16];
+        tmem_ld16<kQuad>(chunk_addr(0), v[0]);
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
+        for (int c = 0; c < kChunks; ++c) {
+          tmem_wait_ld(v[c & 1]);
+          if (c + 1 < kChunks) tmem_ld16<kQuad>(chunk_addr(c + 1), v[(c + 1) & 1]);
+          float *a = acc + 16 * c;
+          const uint32_t(&w)[16] = v[c & 1];
 #pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-              float v[16];
-              tmem_ld16x256b_x4(taddr + ((uint32_t)(16 * h) << 16) + cc * 32, v);
-              float *a = acc + 64 * h + 16 * cc;
-#pragma unroll
-              for (int c = 0; c < 4; ++c) {
-                fma2(a[4 * c], a[4 * c + 1], f[2 * h], v[4 * c], v[4 * c + 1]);
-                fma2(a[4 * c + 2], a[4 * c + 3], f[2 * h + 1], v[4 * c + 2], v[4 * c + 3]);
-              }
-            }
-          }
-        } else {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            float v[32];
-            tmem_ld32(taddr + c * 32, v);
-#pragma unroll
-            for (int i = 0; i < 32; i += 2) fma2(acc[c * 32 + i], acc[c * 32 + i + 1], f[0], v[i], v[i + 1]);
+          for (int i = 0; i < 16; i += 2) {
+            const float fi = f[kQuad ? 2 * (c / (NT / 32)) + ((i >> 1) & 1) : 0];
+            fma2(a[i], a[i + 1], fi, __uint_as_float(w[i]), __uint_as_float(w[i + 1]));
           }
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&acc_empty[buf]);
-        ++bcount;
+        if (lane == 0) mbar_arrive(&acc_empty[accr.s]);
+        accr.next(ntile);
       }
-      // Epilogue: columns are tokens m0 + i, this thread's row is `row`.
-      if (kMode == 0) {
+      if constexpr (kMode == 0) {
+        // Columns are tokens m0 + i, this thread's row is `row`.
+        const int64_t row = vt * kTileRows + rt0;
         if (row < p.V) {
-          const int mcount = p.M - m0 < 128 ? p.M - m0 : 128;  // tokens of this column half inside M
+          const int mcount = p.M - m0 < NT ? p.M - m0 : NT;
           if (p.out_fp32) {
             float *o = reinterpret_cast<float *>(p.out) + (int64_t)m0 * p.V + row;
 #pragma unroll
-            for (int i = 0; i < 128; ++i, o += p.V)
+            for (int i = 0; i < NT; ++i, o += p.V)
               if (i < mcount) *o = acc[i];
           } else {
             __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(p.out) + (int64_t)m0 * p.V + row;
 #pragma unroll
-            for (int i = 0; i < 128; ++i, o += p.V)
+            for (int i = 0; i < NT; ++i, o += p.V)
               if (i < mcount) *o = __float2bfloat16_rn(acc[i]);
           }
         }
-      } else if (kMode == 2) {
-        // Greedy partials: the largest logit of each token over the warp's 32
-        // rows and its row (the lowest on ties).  Layout as for the cross
-        // entropy below: rows rbase + ru + 8 kr of the 32 token columns
-        // col(k) = 8 (k >> 1) + 2 cq + (k & 1); first over the thread's 4
-        // rows (ascending, so the first maximum wins), then a butterfly over
-        // lane bits 4, 3, 2 that halves the column set per step.
-        const int rbase = vt * kTileRows + lg * 32;
-        const int ru = lane >> 2, cq = lane & 3;
-        if (rbase + 32 > p.V) {
-#pragma unroll
-          for (int i = 0; i < 128; ++i) {
-            const int kr = 2 * (i >> 6) + ((i >> 1) & 1);
-            if (rbase + ru + 8 * kr >= p.V) acc[i] = -INFINITY;
-          }
-        }
-        float bv[32];
-        int bi[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const int i0 = 4 * (k >> 1) + (k & 1);
-          const int r = rbase + ru;
-          float v = acc[i0];
-          int ix = r;
-          if (acc[i0 + 2] > v) v = acc[i0 + 2], ix = r + 8;
-          if (acc[i0 + 64] > v) v = acc[i0 + 64], ix = r + 16;
-          if (acc[i0 + 66] > v) v = acc[i0 + 66], ix = r + 24;
-          bv[k] = v;
-          bi[k] = ix;
-        }
-#pragma unroll
-        for (int n = 32, o = 16; n > 4; n >>= 1, o >>= 1) {
-          const bool up = lane & o;
-#pragma unroll
-          for (int j = 0; j < n / 2; ++j) {
-            const float kv = up ? bv[j + n / 2] : bv[j];
-            const int ki = up ? bi[j + n / 2] : bi[j];
-            const float gv = up ? bv[j] : bv[j + n / 2];
-            const int gi = up ? bi[j] : bi[j + n / 2];
-            const float rv = __shfl_xor_sync(0xffffffffu, gv, o);
-            const int ri = __shfl_xor_sync(0xffffffffu, gi, o);
-            const bool take = rv > kv || (rv == kv && ri < ki);
-            bv[j] = take ? rv : kv;
-            bi[j] = take ? ri : ki;
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int m = m0 + 16 * ru + 8 * (j >> 1) + 2 * cq + (j & 1);
-          if (m < p.M) p.ce_part[((int64_t)vt * 4 + lg) * p.M + m] = make_float2(bv[j], __int_as_float(bi[j]));
-        }
       } else {
-        // Layout (see the promotion): this thread holds rows rbase + ru + 8 kr
-        // (kr = 0..3) of 32 token columns col(k) = 8 (k >> 1) + 2 cq + (k & 1),
-        // k = 0..31, row kr of column k at acc[i0(k) + {0, 2, 64, 66}[kr]].
-        const int64_t rbase = (int64_t)vt * kTileRows + lg * 32;
-        const int ru = lane >> 2, cq = lane & 3;
-        // Target logits first: a token whose target is one of this warp's 32
-        // rows takes its value from the thread holding it (rare: about one
-        // token in 37 per warp and tile, so the slow path is a warp-uniform
-        // branch).  Lane (ru, cq) reads the targets of the columns it ends
-        // with: 16 ru + 8 (j >> 1) + 2 cq + (j & 1), j = 0..3.
-        int tg[4];
-        bool hit = false;
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int m = m0 + 16 * ru + 8 * (j >> 1) + 2 * cq + (j & 1);
-          const int64_t t64 = m < p.M ? (int64_t)p.targets[m] - p.row0 - rbase : -1;  // row within the warp's 32
-          tg[j] = t64 >= 0 && t64 < 32 ? (int)t64 : -1;
-          hit |= tg[j] >= 0;
-        }
-        if (__any_sync(0xffffffffu, hit)) {
-#pragma unroll
-          for (int col = 0; col < 128; ++col) {
-            const int j = 2 * ((col >> 3) & 1) + (col & 1);
-            const int owner = 4 * (col >> 4) + ((col >> 1) & 3);  // lane that read this column's target
-            const int r = __shfl_sync(0xffffffffu, tg[j], owner);
-            if (r >= 0) {  // warp-uniform
-              const int i0 = 4 * (col >> 3) + (col & 1);
-              const float mine = r & 16 ? (r & 8 ? acc[i0 + 66] : acc[i0 + 64]) : (r & 8 ? acc[i0 + 2] : acc[i0]);
-              const float v = __shfl_sync(0xffffffffu, mine, 4 * (r & 7) + ((col >> 1) & 3));
-              if (lane == owner) p.ce_tlogit[m0 + col] = v * kLn2;
-            }
-          }
-        }
-        // Rows past V (last tile only) enter as -FLT_MAX: weight 0 against any
-        // logit, and a finite (max, count) when the warp holds no real row.
-        if (rbase + 32 > p.V) {
-#pragma unroll
-          for (int i = 0; i < 128; ++i) {
-            const int kr = 2 * (i >> 6) + ((i >> 1) & 1);
-            if (rbase + ru + 8 * kr >= p.V) acc[i] = -FLT_MAX;
-          }
-        }
-        // (max, sum of 2^(y - max)) of each column over the thread's 4 rows...
-        float mx[32], sm[32];
-#pragma unroll
-        for (int k = 0; k < 32; ++k) {
-          const int i0 = 4 * (k >> 1) + (k & 1);
-          const float v0 = acc[i0], v1 = acc[i0 + 2], v2 = acc[i0 + 64], v3 = acc[i0 + 66];
-          const float mk = fmaxf(fmaxf(v0, v1), fmaxf(v2, v3));
-          mx[k] = mk;
-          sm[k] = (ex2_approx(v0 - mk) + ex2_approx(v1 - mk)) + (ex2_approx(v2 - mk) + ex2_approx(v3 - mk));
-        }
-        // ...then over the 8 lanes with the same lane % 4 (lane bits 4, 3, 2)
-        // by a butterfly that halves the column set per step: the lane with
-        // bit o set keeps the upper half and merges the partner's copy of it.
-        // Lane (ru, cq) ends with k = 4 ru + j, j = 0..3.
-#pragma unroll
-        for (int n = 32, o = 16; n > 4; n >>= 1, o >>= 1) {
-          const bool up = lane & o;
-#pragma unroll
-          for (int j = 0; j < n / 2; ++j) {
-            const float km = up ? mx[j + n / 2] : mx[j], ks = up ? sm[j + n / 2] : sm[j];
-            const float gm = up ? mx[j] : mx[j + n / 2], gs = up ? sm[j] : sm[j + n / 2];
-            const float rm = __shfl_xor_sync(0xffffffffu, gm, o), rs = __shfl_xor_sync(0xffffffffu, gs, o);
-            lse2_merge(km, ks, rm, rs, mx[j], sm[j]);
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int m = m0 + 16 * ru + 8 * (j >> 1) + 2 * cq + (j & 1);
-          if (m < p.M) p.ce_part[((int64_t)vt * 4 + lg) * p.M + m] = make_float2(mx[j] * kLn2, sm[j]);
+        const int64_t rbase = vt * kTileRows + lg * 32, part = vt * 4 + lg;
+        if constexpr (kMode == 2) {
+          quad_argmax<NT, 0>(p, acc, rbase, part, m0, lane);
+          if constexpr (NT == 128) quad_argmax<NT, 1>(p, acc, rbase, part, m0, lane);
+        } else {
+          quad_ce<NT, 0>(p, acc, rbase, part, m0, lane);
+          if constexpr (NT == 128) quad_ce<NT, 1>(p, acc, rbase, part, m0, lane);
         }
       }
     }
@@ -668,36 +944,53 @@ done:
 // ------------------------------------------------------------------------
 // Host side: tensor maps and launch.
 // ------------------------------------------------------------------------
+template <int NT, int kMode, bool kSC4>
+cudaError_t launch_prefill_t(const PrefillParams &p, int grid, bool pdl, cudaStream_t s) {
+  auto kern = prefill_kernel<NT, kMode, kSC4>;
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(kern), PfGeom<NT>::kSmem);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(kPfThreads);
+  cfg.dynamicSmemBytes = PfGeom<NT>::kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, p);
+}
+
 // One packed format's kernel instances (INT8 in prefill.cu, SC4 in prefill_sc4.cu).
 template <bool kSC4>
 cudaError_t launch_prefill_fmt(const archead_pack *pk, const void *x, int M, const uint16_t *T, void *out,
                                int out_fp32, bool argmax, const int32_t *targets, int row0, float2 *ce_part,
-                               float *ce_tlogit, cudaStream_t s) {
+                               float *ce_tlogit, bool pdl, cudaStream_t s) {
   PrefillParams p{};
-  if (!make_tma_map_bf16(&p.tmap_x, x, M, pk->d, 128)) return cudaErrorInvalidValue;
-  const int kt = 2 * (pk->rcp + pk->rrp);
-  if (kt > 0) {
-    if (!make_tma_map_bf16(&p.tmap_t, T, M, kt, 128)) return cudaErrorInvalidValue;
-  }
+  // An MMA of up to 128 tokens costs the same whatever its width, so tiles
+  // are 128 tokens; 64 where all tokens fit (smaller x copies, half the
+  // promotion, deeper rings).
+  const int nt = M <= 64 ? 64 : 128;
+  if (!make_tma_map_bf16(&p.tmap_x, x, M, pk->d, nt)) return cudaErrorInvalidValue;
+  if (pk->lr > 0 && !make_tma_map_bf16(&p.tmap_t, T, M, 2 * pk->lr, nt)) return cudaErrorInvalidValue;
   p.codes = pk->codes;
   p.scales = pk->scales;
   p.scodes = pk->scodes;
   p.s_row = pk->s_row;
-  p.sc4 = pk->sc4;
   p.G_pad2 = pk->G_pad2;
   p.lr_codes = pk->lr_codes;
   p.s_a = pk->s_a;
   p.V = pk->V;
   p.M = M;
   p.num_vt = pk->num_tiles;
-  p.num_mt = (M + kPfN - 1) / kPfN;
+  p.num_mt = (M + nt - 1) / nt;
   p.d_pad = pk->d_pad;
   p.G_pad = pk->G_pad;
   p.g = pk->g;
+  p.blk_log2 = kSC4 ? kSc4BlockLog2 : __builtin_ctz(pk->g) - 4;
   p.nls = pk->nls;
   p.nls_core = pk->nls_core;
-  p.rcp = pk->rcp;
-  p.rrp = pk->rrp;
   p.out = out;
   p.out_fp32 = out_fp32;
   p.targets = targets;
@@ -706,22 +999,24 @@ cudaError_t launch_prefill_fmt(const archead_pack *pk, const void *x, int M, con
   p.ce_tlogit = ce_tlogit;
   p.err = pk->err;
   p.wait_budget = pk->wait_budget;
-  const int tiles = p.num_vt * p.num_mt;
-  const int grid = tiles < pk->sm_count ? tiles : pk->sm_count;
-  if (out) {
-    cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(prefill_kernel<0, kSC4>), kPfSmem);
-    if (e != cudaSuccess) return e;
-    prefill_kernel<0, kSC4><<<grid, kPfThreads, kPfSmem, s>>>(p);
-  } else if (argmax) {
-    cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(prefill_kernel<2, kSC4>), kPfSmem);
-    if (e != cudaSuccess) return e;
-    prefill_kernel<2, kSC4><<<grid, kPfThreads, kPfSmem, s>>>(p);
-  } else {
-    cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(prefill_kernel<1, kSC4>), kPfSmem);
-    if (e != cudaSuccess) return e;
-    prefill_kernel<1, kSC4><<<grid, kPfThreads, kPfSmem, s>>>(p);
-  }
-  return cudaGetLastError();
+  // Two tiles a unit unless one tile a unit leaves the blocks fewer tiles to
+  // do (few units: small heads).
+  const auto rounds = [&](int tl) {
+    const int64_t units = (int64_t)((p.num_vt + tl - 1) / tl) * p.num_mt;
+    return (units + pk->sm_count - 1) / pk->sm_count * tl;
+  };
+  p.tl = 4 * rounds(1) < 3 * rounds(2) ? 1 : 2;
+  const int64_t units = (int64_t)((p.num_vt + p.tl - 1) / p.tl) * p.num_mt;
+  if (units > 0x7fffffff - pk->sm_count) return cudaErrorInvalidValue;
+  const int grid = (int)(units < pk->sm_count ? units : pk->sm_count);
+  const int mode = out ? 0 : argmax ? 2 : 1;
+  if (nt == 64)
+    return mode == 0   ? launch_prefill_t<64, 0, kSC4>(p, grid, pdl, s)
+           : mode == 1 ? launch_prefill_t<64, 1, kSC4>(p, grid, pdl, s)
+                       : launch_prefill_t<64, 2, kSC4>(p, grid, pdl, s);
+  return mode == 0   ? launch_prefill_t<128, 0, kSC4>(p, grid, pdl, s)
+         : mode == 1 ? launch_prefill_t<128, 1, kSC4>(p, grid, pdl, s)
+                     : launch_prefill_t<128, 2, kSC4>(p, grid, pdl, s);
 }
 
 

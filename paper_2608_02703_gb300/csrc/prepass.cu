@@ -31,6 +31,10 @@ __device__ __forceinline__ uint16_t f32_to_bf16_bits(float v) {
   return __bfloat16_as_ushort(__float2bfloat16_rn(v));
 }
 
+// Column of the prefill operand T holding the hi part of extended column kk
+// (its lo part follows 16 columns on): per 16-wide step, 16 hi, 16 lo.
+__device__ __forceinline__ int t_col(int kk) { return 32 * (kk >> 4) + (kk & 15); }
+
 // Shared memory of one block for mt tokens: the staged x chunk [256][mt+1]
 // (floats, token fastest) and, after it is consumed, the per-warp sums
 // [8][mt][32] in the same space.
@@ -140,15 +144,9 @@ __global__ void __launch_bounds__(256) prepass_kernel(PrepassParams p) {
     const uint16_t lo = f32_to_bf16_bits(t - bf16_lo(hi));
     const int mg = m0 + m;
     if (p.T && m < mt) {
-      uint16_t *row = p.T + (int64_t)mg * (2 * p.lr);
-      if (kk < p.rcp) {
-        row[kk] = hi;
-        row[p.rcp + kk] = lo;
-      } else {
-        const int jj = kk - p.rcp;
-        row[2 * p.rcp + jj] = hi;
-        row[2 * p.rcp + p.rrp + jj] = lo;
-      }
+      uint16_t *row = p.T + (int64_t)mg * (2 * p.lr) + t_col(kk);
+      row[0] = hi;
+      row[16] = lo;
     }
     // Column of the decode layout: the same as kk, or with core and
     // correction back to back (core columns as they are, correction ones
@@ -198,6 +196,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, bool vali
 
 __global__ void __launch_bounds__(128) prepass_t_kernel(PrepassParams p, const uint16_t *__restrict__ lr_t,
                                                         int d_pad) {
+  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");  // as above
   extern __shared__ __align__(16) uint16_t pt_smem[];
   uint16_t *xs = pt_smem;                                    // [stages][64][kPtStride]
   uint16_t *bs = pt_smem + kPtStages * kPtTok * kPtStride;   // [stages][32][kPtStride]
@@ -309,11 +308,9 @@ __global__ void __launch_bounds__(128) prepass_t_kernel(PrepassParams p, const u
         lo2 |= (uint32_t)lo << (16 * h);
       }
       const int kk = c0 + n * 8 + 2 * cq;
-      uint16_t *row = p.T + (int64_t)m * (2 * p.lr);
-      const int hi_col = core ? kk : p.rcp + kk;                 // = 2 rcp + j for the correction
-      const int lo_col = core ? p.rcp + kk : p.rcp + p.rrp + kk;  // = 2 rcp + rrp + j
-      *reinterpret_cast<uint32_t *>(row + hi_col) = hi2;
-      *reinterpret_cast<uint32_t *>(row + lo_col) = lo2;
+      uint16_t *row = p.T + (int64_t)m * (2 * p.lr) + t_col(kk);
+      *reinterpret_cast<uint32_t *>(row) = hi2;
+      *reinterpret_cast<uint32_t *>(row + 16) = lo2;
     }
   }
 }
