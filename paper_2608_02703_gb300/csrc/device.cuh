@@ -210,6 +210,23 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
   return mbar_try_wait_a(smem_u32(bar), parity);
 }
 
+// One probe of three barriers, never suspending the thread: 1 if every one's
+// phase with the given parity is complete.  The probes' latencies overlap.
+__device__ __forceinline__ uint32_t mbar_test3_a(uint32_t bar0, uint32_t ph0, uint32_t bar1, uint32_t ph1, uint32_t bar2,
+                                                 uint32_t ph2) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p, q, r;\n"
+      " mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " mbarrier.test_wait.parity.shared::cta.b64 q, [%3], %4;\n"
+      " mbarrier.test_wait.parity.shared::cta.b64 r, [%5], %6;\n"
+      " and.pred p, p, q;\n and.pred p, p, r;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar0), "r"(ph0), "r"(bar1), "r"(ph1), "r"(bar2), "r"(ph2)
+      : "memory");
+  return ok;
+}
+
 // Bounded wait: spins until the phase with the given parity completed, the
 // block-wide abort flag (if any) is raised, or `budget` clock cycles pass.  On
 // timeout it latches kErrWaitTimeout in *err and raises the abort flag.

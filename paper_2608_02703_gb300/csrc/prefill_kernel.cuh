@@ -2,47 +2,53 @@
 // (paper, Section 3.2, Eq. 7; no dense W_hat is formed, the residual is
 // dequantised tile by tile inside the kernel as Appendix B allows).
 //
-// A unit of work is one or two 128-row vocabulary tiles x NT tokens (64 or
-// 128).  The vocabulary rows are the MMA's M side (one TMEM lane each), the
-// tokens the N side.  Per 64-wide k step:
-//   - one producer warp loads the x tile (NT tokens x 64, bf16, 128-byte
-//     swizzle) by TMA into its ring, another the tiles' 4 KB code chunks into
+// A unit of work is one 128-row vocabulary tile x TM tokens (64, 128 or 256).
+// The vocabulary rows are the MMA's M side (one TMEM lane each), the tokens
+// the N side.  Per stage of 128 of d:
+//   - one producer warp loads the x tiles (up to 128 tokens each, bf16,
+//     128-byte swizzle) by TMA into its ring, another the 8 KB of codes into
 //     theirs, so codes run ahead of x as far as their ring allows;
-//   - a warpgroup per tile turns the codes into exact bf16 integers and stores
-//     them as the A operand in tensor memory: the code layout is that of
-//     m16n8k16 fragments, which is the register layout of tcgen05.st.16x128b;
-//   - one thread issues four tcgen05.mma (kind::f16, 128 x NT x 16, A from
-//     TMEM, B = x from shared memory, fp32 accumulate) per tile into a ring of
-//     TMEM accumulators.  The two tiles take turns, so each x slot feeds two
-//     tiles and one tile's finished group is drained while the other computes;
-//   - a warpgroup per tile reads each finished block with tcgen05.ld and adds
+//   - a converter warpgroup (two or four take stages in turn) turns the codes
+//     into exact bf16 integers and stores them as the A operand in tensor
+//     memory: the code layout is that of m16n8k16 fragments, which is the
+//     register layout of tcgen05.st.16x128b;
+//   - one thread issues eight tcgen05.mma (kind::f16, 128 x 64 or 128 x 16, A
+//     from TMEM, B = x from shared memory, fp32 accumulate) into a ring of
+//     TMEM accumulators; with 256 tokens, eight for each half of them, so that
+//     each conversion serves 256 tokens and one half's finished group is
+//     drained while the other computes;
+//   - promotion warps read each finished block with tcgen05.ld and add
 //     s[row, group] * partial to fp32 registers (group-wise scales cannot be
 //     folded into exact bf16 operands).
-// The rank-r branches are further k steps: 32 columns of int8 codes of A_c
-// (factor 1) or A_w (factor = row scale of A_w), each 16 of them multiplied
-// with the bf16 hi and lo parts of the pre-pass's t, read through a second
-// tensor map.
+// The rank-r branches are further k steps: 64 columns of int8 codes of A_c
+// (factor 1) or A_w (factor = row scale of A_w) a stage, each 16 of them
+// multiplied with the bf16 hi and lo parts of the pre-pass's t, read through a
+// second tensor map.
 //
 // In the paper's packed format (SC4) a group scale is s_row * (q + 1) with a
 // 4-bit code q.  The converters fold q + 1 into the operand (code * (q + 1)
 // stays an exact bf16 integer, |.| <= 128), and blocks are 512 wide,
 // promoted by s_row.
 //
-// Why A in tensor memory and two tiles a unit: with A and x in shared memory
-// a 128 x 256 x 16 MMA reads 12 KB in its 128 cycles, the x copy of a k step
-// writes 32 KB and the converters 16 KB, together more than the 128 bytes a
-// cycle shared memory moves; that arrangement ran at 62 % of the measured
-// tensor peak.  Here the MMAs of a k step and tile read 16 KB of x, written
-// once for two tiles, in about 280 cycles.  An MMA of at most 128 tokens takes
-// 69-74 cycles whatever its width, so 17 to 128 tokens cost one pass over the
-// head (measured for the Qwen3-8B shape in the launch rule below).
+// What bounds it.  With A and x in shared memory (the earlier form of this
+// kernel) a 128 x 256 x 16 MMA reads 12 KB in its 128 cycles, the x copy of a
+// 64-wide k step writes 32 KB and the converters 16 KB: together more than the
+// 128 bytes a cycle that shared memory moves, and it ran at 62 % of the
+// measured tensor peak.  With A in TMEM an MMA of N tokens takes about N / 2 +
+// 5 cycles (measured alone: 39 for 64, 67 for 128), and what is left is the
+// issuing warp's own instructions (two turns a stage: about 1350 cycles, 1070
+// of them MMAs) and, below 129 tokens, the conversion of the codes, which does
+// not depend on the tokens.  Qwen3-8B shape, start and now: 24 tokens 150 ->
+// 142 us, 64 tokens 246 -> 149, 4096 tokens 4.47 -> 3.72 ms; the paper's
+// format 200 tokens 319 -> 220 us, cross entropy of 2048 tokens 2.14 -> 1.72
+// ms; Gemma shape, cross entropy of 512 tokens 781 -> 684 us.
 //
 // Epilogues: logits (each promotion thread stores one row of its tokens),
 // greedy partials (largest logit and its row per token over each warp's 32
 // rows) and cross-entropy partials (max and sum of exp per token over each
 // warp's 32 rows, plus the target's logit).  The cross-entropy and greedy
 // instances read TMEM in the 16x256b shape, so that a thread holds 4 rows
-// of NT / 4 tokens and most of the reduction over rows is thread-local.
+// of a quarter of them and most of the reduction over rows is thread-local.
 #pragma once
 
 #include <cfloat>
@@ -53,37 +59,51 @@
 
 namespace archead {
 
-constexpr int kPfThreads = 640;  // producers + MMA, two converter and two promotion warpgroups
 constexpr int kPfTmemCols = 512;
 constexpr float kLog2e = 1.4426950408889634f;  // log2(e)
 constexpr float kLn2 = 0.6931471805599453f;    // ln(2)
 
-// Shared-memory rings and TMEM columns for NT tokens a tile.  A stage is 128
-// of d (or four 16-wide rank-r steps).  TMEM: kNB accumulators of NT columns,
-// then two rings (one a converter warpgroup) of kAS A stages (128 rows x 128
-// k, two halves of 32 columns).
-template <int NT>
+// Instance geometry for TM tokens a unit, in kH halves of NT.  A stage is 128
+// of d (or four 16-wide rank-r steps); x slots hold one half's.  TMEM: kNB
+// accumulators of NT columns, then one A stage (128 rows x 128 k, 64 columns)
+// a converter warpgroup.  Up to 128 tokens conversion is most of the work (it
+// does not depend on the tokens): four converter warpgroups; 256 tokens need
+// the registers for 128 accumulators a promotion thread.
+template <int TM>
 struct PfGeom {
-  static constexpr int kBoxBytes = NT * 64 * 2;  // one TMA box of x: 64 of d
-  static constexpr int kXBytes = 2 * kBoxBytes;
-  static constexpr int kXStages = NT == 128 ? 4 : 5;
-  static constexpr int kScaleOff = 4 * kChunkBytes;  // SC4: up to two byte rows of scale codes a tile
-  static constexpr int kCodeSlot = kScaleOff + 4 * kTileRows;
-  static constexpr int kCodeStages = NT == 128 ? 5 : 7;
-  static constexpr int kNB = NT == 128 ? 3 : 4;
-  static constexpr int kAS = NT == 128 ? 1 : 2;
+  static constexpr int NT = TM == 64 ? 64 : 128;
+  static constexpr int kH = TM / NT;
+  static constexpr int kConv = TM == 256 ? 2 : 4;    // converter warpgroups
+  static constexpr int kPromo = TM == 64 ? 1 : 2;    // promotion warpgroups
+  static constexpr int kCols = TM == 256 ? 128 : 64; // accumulator columns a promotion thread holds
+  static constexpr int kThreads = 128 * (1 + kConv + kPromo);
+  static constexpr int kNB = TM == 64 ? 4 : TM == 128 ? 2 : 3;
   static constexpr int kABase = kNB * NT;
-  static constexpr int kCodeOff = kXStages * kXBytes;
-  static constexpr int kBarOff = kCodeOff + kCodeStages * kCodeSlot;
-  static constexpr int kBars = 3 * kXStages + 2 * kCodeStages + 4 * kAS + 2 * kNB + 1;
+  static constexpr int kAParts = TM == 256 ? 2 : 1;  // an A stage is released in parts (256 tokens: halves)
+  static constexpr int kBoxBytes = NT * 64 * 2;      // one TMA box of x: 64 of d
+  static constexpr int kXBytes = 2 * kBoxBytes;
+  static constexpr int kXS = TM == 64 ? 8 : TM == 128 ? 5 : 5;
+  static constexpr int kScaleOff = 2 * kChunkBytes;  // SC4: up to two byte rows of scale codes
+  static constexpr int kCodeSlot = kScaleOff + 2 * kTileRows;
+  static constexpr int kCS = TM == 64 ? 11 : TM == 128 ? 7 : 7;
+  static constexpr int kCodeOff = kXS * kXBytes;
+  static constexpr int kBarOff = kCodeOff + kCS * kCodeSlot;
+  static constexpr int kBars = 2 * kXS + 2 * kCS + kConv * (1 + kAParts) + 2 * kNB + 1;
   static constexpr int kSmem = 1024 + kBarOff + kBars * 8 + 16;
-  static_assert(kABase + 2 * kAS * 64 <= kPfTmemCols, "TMEM columns");
+  // Registers a thread of the producer/MMA warpgroup, the converters and the
+  // promotion warpgroups (launched with the largest multiple of 8 that fits);
+  // their sum is that of the launch.
+  static constexpr int kRegs0 = TM == 256 ? 48 : 56;
+  static constexpr int kRegsC = TM == 64 ? 72 : 56;
+  static constexpr int kRegsP = TM == 64 ? 128 : TM == 128 ? 112 : 160;
+  static_assert(128 * (kRegs0 + kConv * kRegsC + kPromo * kRegsP) <= 65536 / kThreads / 8 * 8 * kThreads, "registers");
+  static_assert(kABase + kConv * 64 <= kPfTmemCols, "TMEM columns");
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
 
 struct PrefillParams {
-  CUtensorMap tmap_x;   // bf16 [M][d], box 64 x NT, 128B swizzle
-  CUtensorMap tmap_t;   // bf16 [M][2*LR], box 64 x NT, 128B swizzle
+  CUtensorMap tmap_x;   // bf16 [M][d], box 64 x nt, 128B swizzle
+  CUtensorMap tmap_t;   // bf16 [M][2*LR], box 64 x nt, 128B swizzle
   const uint8_t *codes;
   const uint16_t *scales;  // fp16 group scales (INT8 format)
   const uint8_t *scodes;   // 4-bit group-scale codes (SC4 format)
@@ -91,7 +111,8 @@ struct PrefillParams {
   const uint8_t *lr_codes;
   const uint16_t *s_a;
   int64_t V;
-  int M, num_vt, num_mt, tl, d_pad, G_pad, g, nls, nls_core;  // tl: vocabulary tiles per unit (1 or 2)
+  int M, num_vt, num_mt, d_pad, G_pad, g, nls, nls_core;
+  int nt;  // tokens of an MMA and of an x box, a multiple of 16 up to the instance's NT
   int G_pad2;
   int blk_log2;  // log2 of a residual block's 16-wide steps (g / 16; SC4: kSc4BlockSteps)
   void *out;
@@ -295,8 +316,8 @@ __device__ __forceinline__ constexpr int quad_i0(int k) {
 
 // Greedy partials: the largest logit of each token and its row (lowest on ties).
 template <int NT, int HH>
-__device__ __forceinline__ void quad_argmax(const PrefillParams &p, const float (&acc)[NT], int64_t rbase, int64_t part,
-                                            int m0, int lane) {
+__device__ __forceinline__ void quad_argmax(const PrefillParams &p, const float (&acc)[NT], int64_t rbase, int64_t part, int m0,
+                                            int mend, int lane) {
   const int ru = lane >> 2, cq = lane & 3;
   const int valid = rbase + 32 > p.V ? (int)(p.V - rbase) : 32;  // rows of the warp inside V
   float bv[16];
@@ -331,7 +352,7 @@ __device__ __forceinline__ void quad_argmax(const PrefillParams &p, const float 
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int m = m0 + 64 * HH + 8 * ru + 2 * cq + j;
-    if (m < p.M) p.ce_part[part * p.M + m] = make_float2(bv[j], __int_as_float((int)rbase + bi[j]));
+    if (m < mend) p.ce_part[part * p.M + m] = make_float2(bv[j], __int_as_float((int)rbase + bi[j]));
   }
 }
 
@@ -339,7 +360,7 @@ __device__ __forceinline__ void quad_argmax(const PrefillParams &p, const float 
 // target's logit.  The accumulators are in units of ln 2.
 template <int NT, int HH>
 __device__ __forceinline__ void quad_ce(const PrefillParams &p, float (&acc)[NT], int64_t rbase, int64_t part, int m0,
-                                        int lane) {
+                                            int mend, int lane) {
   const int ru = lane >> 2, cq = lane & 3;
   m0 += 64 * HH;
   // Target logits first: a token whose target is one of this warp's 32 rows
@@ -351,7 +372,7 @@ __device__ __forceinline__ void quad_ce(const PrefillParams &p, float (&acc)[NT]
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int m = m0 + 8 * ru + 2 * cq + j;
-    const int64_t t64 = m < p.M ? (int64_t)p.targets[m] - p.row0 - rbase : -1;  // row within the warp's 32
+    const int64_t t64 = m < mend ? (int64_t)p.targets[m] - p.row0 - rbase : -1;  // row within the warp's 32
     tg[j] = t64 >= 0 && t64 < 32 ? (int)t64 : -1;
     hit |= tg[j] >= 0;
   }
@@ -404,27 +425,26 @@ __device__ __forceinline__ void quad_ce(const PrefillParams &p, float (&acc)[NT]
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int m = m0 + 8 * ru + 2 * cq + j;
-    if (m < p.M) p.ce_part[part * p.M + m] = make_float2(mx[j] * kLn2, sm[j]);
+    if (m < mend) p.ce_part[part * p.M + m] = make_float2(mx[j] * kLn2, sm[j]);
   }
 }
 
-// NT: tokens per tile; kMode 0: logits, 1: cross-entropy partials, 2: greedy
+// TM: tokens per unit; kMode 0: logits, 1: cross-entropy partials, 2: greedy
 // (largest logit, row) partials; kSC4: the paper's packed format (group-scale
 // codes times row scales).
-template <int NT, int kMode, bool kSC4>
-__global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_constant__ PrefillParams p) {
-  using G = PfGeom<NT>;
-  constexpr int kNB = G::kNB, kAS = G::kAS, kXS = G::kXStages;
+template <int TM, int kMode, bool kSC4>
+__global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const __grid_constant__ PrefillParams p) {
+  using G = PfGeom<TM>;
+  constexpr int NT = G::NT, kNB = G::kNB, kXS = G::kXS, kCS = G::kCS, kConv = G::kConv, kCols = G::kCols;
   extern __shared__ uint8_t pf_smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
-  // ready[t][x slot]: tile t's A stage is converted and, for t = 0, x has
-  // landed (tile 1's MMAs of a stage follow tile 0's).
-  uint64_t *ready = reinterpret_cast<uint64_t *>(smem + G::kBarOff);
-  uint64_t *x_empty = ready + 2 * kXS;
+  uint64_t *x_full = reinterpret_cast<uint64_t *>(smem + G::kBarOff);
+  uint64_t *x_empty = x_full + kXS;
   uint64_t *c_full = x_empty + kXS;
-  uint64_t *c_empty = c_full + G::kCodeStages;
-  uint64_t *a_empty = c_empty + G::kCodeStages;  // [2][kAS][half]
-  uint64_t *acc_full = a_empty + 4 * kAS;
+  uint64_t *c_empty = c_full + kCS;
+  uint64_t *a_full = c_empty + kCS;
+  uint64_t *a_empty = a_full + kConv;  // [kConv][kAParts]
+  uint64_t *acc_full = a_empty + kConv * G::kAParts;
   uint64_t *acc_empty = acc_full + kNB;
   uint64_t *drain = acc_empty + kNB;
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(drain + 1);
@@ -434,7 +454,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
   const int KC = p.d_pad / 128;      // residual stages
   const int KE = (p.nls + 3) / 4;    // rank-r stages of four 16-wide steps (the last: two or four)
   const int KS = KC + KE;
-  const int num_units = (p.num_vt + p.tl - 1) / p.tl * p.num_mt;
+  const int num_units = p.num_vt * p.num_mt;
   // Promotion blocks of a tile: residual blocks, then the core and the
   // correction branches.
   const int nres = ((KC * 8 - 1) >> p.blk_log2) + 1;
@@ -442,10 +462,11 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
   const int nb = nres + has_core + has_corr;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kXS; ++i) mbar_init(&ready[i], 5), mbar_init(&ready[kXS + i], 4), mbar_init(&x_empty[i], 1);
-    for (int i = 0; i < G::kCodeStages; ++i) mbar_init(&c_full[i], 1), mbar_init(&c_empty[i], 8);
-    for (int i = 0; i < 4 * kAS; ++i) mbar_init(&a_empty[i], 1);
-    for (int i = 0; i < kNB; ++i) mbar_init(&acc_full[i], 1), mbar_init(&acc_empty[i], 4);
+    for (int i = 0; i < kXS; ++i) mbar_init(&x_full[i], 1), mbar_init(&x_empty[i], 1);
+    for (int i = 0; i < kCS; ++i) mbar_init(&c_full[i], 1), mbar_init(&c_empty[i], 4);
+    for (int i = 0; i < kConv; ++i) mbar_init(&a_full[i], 4);
+    for (int i = 0; i < kConv * G::kAParts; ++i) mbar_init(&a_empty[i], 1);
+    for (int i = 0; i < kNB; ++i) mbar_init(&acc_full[i], 1), mbar_init(&acc_empty[i], TM == 128 ? 8 : 4);
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
@@ -457,72 +478,64 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
   const uint32_t tmem_base = *tmem_slot;
   bool mma_leader = false;  // the lane of warp 1 that issues the MMAs
 
-  // Registers are rebalanced between warpgroups (launch: 640 x 96).  128
-  // accumulators a promotion thread leave 160 for those warpgroups, 56 for
-  // the converters, 48 for producers and MMA: 128 * 48 + 256 * 56 + 256 * 160
-  // = 640 * 96; with 64 accumulators 128, 64 and 56.  Each role's code follows
-  // its own setmaxnreg so that the compiler allocates within that budget.
+  // Registers are rebalanced between warpgroups (PfGeom).  Each role's code
+  // follows its own setmaxnreg so that the compiler allocates within that budget.
   if (warp < 4) {
-    if constexpr (NT == 128)
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 48;\n" ::: "memory");
-    else
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;\n" ::: "memory");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(G::kRegs0) : "memory");
     if (warp == 0) {
       // ------------------------------ x producer ------------------------------
       // The whole warp runs the loop (uniform waits); one elected lane issues.
       const bool leader = elect_one();
       RingPos<kXS> r;
       int issued = 0;
+      bool t_ready = false;
       for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
-        const int m0 = (u % p.num_mt) * NT;
+        const int m0 = (u % p.num_mt) * (G::kH * p.nt);
         for (int e = 0; e < KS; ++e) {
-          if (!mbar_wait_warp(&x_empty[r.s], r.ph ^ 1, p.wait_budget, abort_flag, p.err)) {
-            drain_copies(ready, kXS, issued, p.wait_budget, p.err);
-            goto done;
+          if (e == KC && !t_ready) {
+            asm volatile("griddepcontrol.wait;\n" ::: "memory");  // t comes from the pre-pass grid
+            t_ready = true;
           }
-          if (e == KC && issued < KS) asm volatile("griddepcontrol.wait;\n" ::: "memory");  // t is the pre-pass grid's
-          if (leader) {
-            uint8_t *dst = smem + r.s * G::kXBytes;
-            if (e < KC) {
-              mbar_arrive_expect_tx(&ready[r.s], G::kXBytes);
-              tma_load_2d(dst, &p.tmap_x, e * 128, m0, &ready[r.s]);
-              tma_load_2d(dst + G::kBoxBytes, &p.tmap_x, e * 128 + 64, m0, &ready[r.s]);
-            } else {
-              const bool two = 4 * (e - KC) + 2 < p.nls;
-              mbar_arrive_expect_tx(&ready[r.s], two ? G::kXBytes : G::kBoxBytes);
-              tma_load_2d(dst, &p.tmap_t, (e - KC) * 128, m0, &ready[r.s]);
-              if (two) tma_load_2d(dst + G::kBoxBytes, &p.tmap_t, (e - KC) * 128 + 64, m0, &ready[r.s]);
+          for (int t = 0; t < G::kH; ++t) {
+            if (!mbar_wait_warp(&x_empty[r.s], r.ph ^ 1, p.wait_budget, abort_flag, p.err)) {
+              drain_copies(x_full, kXS, issued, p.wait_budget, p.err);
+              goto done;
             }
+            if (leader) {
+              uint8_t *dst = smem + r.s * G::kXBytes;
+              const CUtensorMap *map = e < KC ? &p.tmap_x : &p.tmap_t;
+              const int c = (e < KC ? e : e - KC) * 128;
+              const bool two = e < KC || 4 * (e - KC) + 2 < p.nls;
+              mbar_arrive_expect_tx(&x_full[r.s], (uint32_t)p.nt * (two ? 256 : 128));
+              tma_load_2d(dst, map, c, m0 + t * p.nt, &x_full[r.s]);
+              if (two) tma_load_2d(dst + G::kBoxBytes, map, c + 64, m0 + t * p.nt, &x_full[r.s]);
+            }
+            ++issued;
+            r.next();
+            __syncwarp();
           }
-          ++issued;
-          r.next();
-          __syncwarp();
         }
       }
     } else if (warp == 2) {
       // ------------------------------ code producer ------------------------------
       const bool leader = elect_one();
-      RingPos<G::kCodeStages> r;
+      RingPos<kCS> r;
       int issued = 0;
       const int lg = __ffs(p.g) - 1;
       const uint32_t scale_bytes = (uint32_t)p.G_pad * kTileRows * 2;
       for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
-        const int vt0 = u / p.num_mt * p.tl;
-        const int ntile = min(p.tl, p.num_vt - vt0);
+        const int64_t vt = u / p.num_mt;
         if (!kSC4 && leader) {
           // The group scales are read by the promotion warps from global
           // memory: bring this block's first and then each next unit's to L2.
-          if (u == (int)blockIdx.x) bulk_prefetch_l2(p.scales + (int64_t)vt0 * p.G_pad * kTileRows, scale_bytes * ntile);
+          if (u == (int)blockIdx.x) bulk_prefetch_l2(p.scales + vt * p.G_pad * kTileRows, scale_bytes);
           const int un = u + (int)gridDim.x;
-          if (un < num_units) {
-            const int vn = un / p.num_mt * p.tl;
-            if (vn != vt0)
-              bulk_prefetch_l2(p.scales + (int64_t)vn * p.G_pad * kTileRows, scale_bytes * min(p.tl, p.num_vt - vn));
-          }
+          if (un < num_units && un / p.num_mt != vt)
+            bulk_prefetch_l2(p.scales + (int64_t)(un / p.num_mt) * p.G_pad * kTileRows, scale_bytes);
         }
         for (int e = 0; e < KS; ++e) {
           if (!mbar_wait_warp(&c_empty[r.s], r.ph ^ 1, p.wait_budget, abort_flag, p.err)) {
-            drain_copies(c_full, G::kCodeStages, issued, p.wait_budget, p.err);
+            drain_copies(c_full, kCS, issued, p.wait_budget, p.err);
             goto done;
           }
           if (leader) {
@@ -530,21 +543,15 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
             if (e < KC) {
               // SC4: the byte rows of scale codes holding this stage's groups.
               const uint32_t sc = kSC4 ? (lg == 5 ? 2 * kTileRows : kTileRows) : 0;
-              mbar_arrive_expect_tx(&c_full[r.s], (uint32_t)ntile * (2 * kChunkBytes + sc));
-              for (int t = 0; t < ntile; ++t) {
-                const int64_t vt = vt0 + t;
-                bulk_g2s(dst + t * 2 * kChunkBytes, p.codes + (vt * KC + e) * 2 * kChunkBytes, 2 * kChunkBytes,
+              mbar_arrive_expect_tx(&c_full[r.s], 2 * kChunkBytes + sc);
+              bulk_g2s(dst, p.codes + (vt * KC + e) * 2 * kChunkBytes, 2 * kChunkBytes, &c_full[r.s]);
+              if (kSC4)
+                bulk_g2s(dst + G::kScaleOff, p.scodes + (vt * p.G_pad2 + ((e * 128) >> lg >> 1)) * kTileRows, sc,
                          &c_full[r.s]);
-                if (kSC4)
-                  bulk_g2s(dst + G::kScaleOff + t * 2 * kTileRows,
-                           p.scodes + (vt * p.G_pad2 + ((e * 128) >> lg >> 1)) * kTileRows, sc, &c_full[r.s]);
-              }
             } else {
               const uint32_t bytes = min(4, p.nls - 4 * (e - KC)) * kLrStepBytes;
-              mbar_arrive_expect_tx(&c_full[r.s], (uint32_t)ntile * bytes);
-              for (int t = 0; t < ntile; ++t)
-                bulk_g2s(dst + t * 2 * kChunkBytes,
-                         p.lr_codes + ((int64_t)(vt0 + t) * p.nls + 4 * (e - KC)) * kLrStepBytes, bytes, &c_full[r.s]);
+              mbar_arrive_expect_tx(&c_full[r.s], bytes);
+              bulk_g2s(dst, p.lr_codes + (vt * p.nls + 4 * (e - KC)) * kLrStepBytes, bytes, &c_full[r.s]);
             }
           }
           ++issued;
@@ -556,57 +563,79 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
       // ------------------------------ MMA issuer ------------------------------
       // As for the producers: the warp runs the loop, one elected lane issues.
       //
-      // The tiles of a unit take turns of at most one stage of a block (one
-      // rank-r step, hi and lo), so that block starts alternate between the
-      // tiles: accumulator i of the ring is the unit's block (i - base) /
-      // ntile of tile (i - base) % ntile.
-      //
-      // This loop's own instructions bound the kernel unless they are few (one
-      // wait per stage and tile): x arrives on the converters' barrier, and
-      // the converters pass a finished stage on to the x producer.
+      // The halves of a unit take turns of at most one stage of a block (one
+      // rank-r step, hi and lo), so that block starts alternate between them:
+      // accumulator i of the ring is the unit's block (i - base) / kH of half
+      // (i - base) % kH.
       const bool leader = elect_one();
       mma_leader = leader;
-      constexpr uint32_t idesc = idesc_bf16(128, NT);
+      const uint32_t idesc = idesc_bf16(128, p.nt);
       const uint64_t xdesc = smem_desc_sw128(smem_u32(smem));
-      const uint32_t ready_a = smem_u32(ready), a_empty_a = smem_u32(a_empty), acc_full_a = smem_u32(acc_full),
-                     acc_empty_a = smem_u32(acc_empty);
-      constexpr uint32_t kBox = G::kBoxBytes >> 4;  // descriptor step to the second box of a stage
+      const uint32_t x_full_a = smem_u32(x_full), x_empty_a = smem_u32(x_empty), a_full_a = smem_u32(a_full),
+                     a_empty_a = smem_u32(a_empty), acc_full_a = smem_u32(acc_full), acc_empty_a = smem_u32(acc_empty);
+      constexpr uint32_t kBox = G::kBoxBytes >> 4;  // descriptor step to the second box of a slot
       RingPos<kXS> xr;
-      RingPos<kAS> ar0, ar1;  // A stages consumed from the converter rings
-      RingPos<kNB> accr;      // next accumulator to start
+      RingPos<kConv> ar;
+      RingPos<kNB> accr;  // next accumulator to start
 
       auto wait = [&](uint32_t bar, uint32_t ph) { return mbar_wait_warp_a(bar, ph, p.wait_budget, abort_flag, p.err); };
       // Starts the next accumulator once it is drained: its columns in d, its barrier in f.
-      auto acc_start = [&](uint32_t &d, uint32_t &f) {
-        if (!wait(acc_empty_a + 8 * accr.s, accr.ph ^ 1)) return false;
+      auto acc_take = [&](uint32_t &d, uint32_t &f) {
         d = tmem_base + accr.s * NT;
         f = acc_full_a + 8 * accr.s;
         accr.next();
+      };
+      auto acc_start = [&](uint32_t &d, uint32_t &f) {
+        if (!wait(acc_empty_a + 8 * accr.s, accr.ph ^ 1)) return false;
+        acc_take(d, f);
         return true;
       };
-      auto ready_wait = [&](int t) { return wait(ready_a + 8 * (t * kXS + xr.s), xr.ph); };
-      // N MMAs from 16-wide step q0 of a residual stage of ring r; first: the
-      // block starts here; f != 0: it ends here.  A half is released after its last step.
-      auto steps = [&](auto n, int q0, int r, const RingPos<kAS> &ar, uint32_t d, bool first, uint32_t f) {
+      // A satisfied mbarrier probe takes ~90 cycles here, and three in a row
+      // before every eight MMAs left the tensor pipe idle.  So the next turn's
+      // barriers are probed together between this turn's MMAs; only a turn
+      // whose probe failed waits.  (Barriers a turn does not need repeat x's.)
+      uint32_t polled = 0;  // this turn's barriers were all seen complete
+      auto poll = [&](const RingPos<kXS> &x, bool need_a, const RingPos<kConv> &a, bool need_acc) {
+        const uint32_t xb = x_full_a + 8 * x.s;
+        polled = mbar_test3_a(xb, x.ph, need_a ? a_full_a + 8 * a.s : xb, need_a ? a.ph : x.ph,
+                              need_acc ? acc_empty_a + 8 * accr.s : xb, need_acc ? accr.ph ^ 1 : x.ph);
+      };
+      // Before a half's first MMAs of a stage: its x, and (first half) the A stage.
+      auto operands = [&](int t, const RingPos<kXS> &x) {
+        return wait(x_full_a + 8 * x.s, x.ph) && (t > 0 || wait(a_full_a + 8 * ar.s, ar.ph));
+      };
+      // N MMAs from 16-wide step q0 of a residual stage; first: the block
+      // starts here; f != 0: it ends here; free_a: no later half reads these A
+      // columns.  With eight, `mid` runs between the first four and the rest.
+      auto steps = [&](auto n, int q0, const RingPos<kXS> &x, uint32_t d, bool first, uint32_t f, bool free_a, auto mid) {
         constexpr int N = decltype(n)::value;
         tc_fence_after();
-        const uint32_t a = tmem_base + G::kABase + (r * kAS + ar.s) * 64 + 8 * q0;
-        const uint32_t ae = a_empty_a + 16 * (r * kAS + ar.s);
-        const uint64_t b = xdesc + (uint32_t)(xr.s * (G::kXBytes >> 4)) + (q0 >> 2) * kBox + 2 * (q0 & 3);
+        const uint32_t a = tmem_base + G::kABase + ar.s * 64 + 8 * q0;
+        const uint32_t ae = a_empty_a + 8 * G::kAParts * ar.s, xe = x_empty_a + 8 * x.s;
+        const uint64_t b = xdesc + (uint32_t)(x.s * (G::kXBytes >> 4)) + (q0 >> 2) * kBox + 2 * (q0 & 3);
         if (leader) {
 #pragma unroll
-          for (int q = 0; q < N; ++q) {  // +2 in the descriptor: 32 bytes in 16-byte units
-            tc_mma_ts(d, a + 8 * q, b + (q >> 2) * kBox + 2 * (q & 3), idesc, q > 0 || !first);
-            if (N >= 4 && (q & 3) == 3) tc_commit_a(ae + 8 * ((q0 + q) >> 2));
+          for (int q = 0; q < (N < 4 ? N : 4); ++q)  // +2 in the descriptor: 32 bytes in 16-byte units
+            tc_mma_ts(d, a + 8 * q, b + 2 * q, idesc, q > 0 || !first);
+          if (q0 + N == 4 || N == 8) {
+            if (G::kAParts == 2 && free_a) tc_commit_a(ae);
           }
-          if (N == 2 && (q0 & 2)) tc_commit_a(ae + 8 * (q0 >> 2));
+        }
+        __syncwarp();
+        mid();
+        if (leader) {
+#pragma unroll
+          for (int q = 4; q < N; ++q) tc_mma_ts(d, a + 8 * q, b + kBox + 2 * (q & 3), idesc, 1);
+          if (q0 + N == 8) {
+            tc_commit_a(xe);
+            if (free_a) tc_commit_a(ae + 8 * (G::kAParts - 1));
+          }
           if (f) tc_commit_a(f);
         }
         __syncwarp();
       };
 
       for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
-        const int ntile = min(p.tl, p.num_vt - u / p.num_mt * p.tl);
         uint32_t d0 = 0, d1 = 0, f0 = 0, f1 = 0;
         if (p.blk_log2 >= 3) {  // blocks of whole stages
           const int per = 1 << (p.blk_log2 - 3);
@@ -616,43 +645,46 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
             if (first) left = per;
             --left;
             const bool last = left == 0 || e + 1 == KC;
-            if (first && !acc_start(d0, f0)) goto done;
-            if (!ready_wait(0)) goto done;
-            if (ntile == 2) {
-              steps(Int<8>{}, 0, 0, ar0, d0, first, last ? f0 : 0);
-              if (first && !acc_start(d1, f1)) goto done;
-              if (!ready_wait(1)) goto done;
-              steps(Int<8>{}, 0, 1, ar1, d1, first, last ? f1 : 0);
-              ar0.next();
-              ar1.next();
-            } else if (e & 1) {
-              steps(Int<8>{}, 0, 1, ar1, d0, first, last ? f0 : 0);
-              ar1.next();
-            } else {
-              steps(Int<8>{}, 0, 0, ar0, d0, first, last ? f0 : 0);
-              ar0.next();
+            if (!__all_sync(0xffffffffu, polled)) {
+              if (first && !wait(acc_empty_a + 8 * accr.s, accr.ph ^ 1)) goto done;
+              if (!operands(0, xr)) goto done;
             }
-            xr.next();
+            if (first) acc_take(d0, f0);
+            if constexpr (G::kH == 2) {
+              const RingPos<kXS> x1 = xr.ahead(1);
+              steps(Int<8>{}, 0, xr, d0, first, last ? f0 : 0, false, [&] { poll(x1, false, ar, first); });
+              if (!__all_sync(0xffffffffu, polled)) {
+                if (first && !wait(acc_empty_a + 8 * accr.s, accr.ph ^ 1)) goto done;
+                if (!operands(1, x1)) goto done;
+              }
+              if (first) acc_take(d1, f1);
+              xr.next(2);
+              steps(Int<8>{}, 0, x1, d1, first, last ? f1 : 0, true, [&] { poll(xr, true, ar.ahead(1), left == 0); });
+            } else {
+              const RingPos<kXS> x0 = xr;
+              xr.next();
+              steps(Int<8>{}, 0, x0, d0, first, last ? f0 : 0, true, [&] { poll(xr, true, ar.ahead(1), left == 0); });
+            }
+            ar.next();
           }
+          polled = 0;  // (the last probe may be of a rank-r stage)
         } else {  // groups of 64 (two blocks a stage) or 32 (four)
           const int nq = p.blk_log2 == 2 ? 4 : 2;
           for (int e = 0; e < KC; ++e) {
             for (int q0 = 0; q0 < 8; q0 += nq) {
-              for (int t = 0; t < ntile; ++t) {
+              for (int t = 0; t < G::kH; ++t) {
+                const RingPos<kXS> x = xr.ahead(t);
                 uint32_t d, f;
                 if (!acc_start(d, f)) goto done;
-                if (q0 == 0 && !ready_wait(t)) goto done;
-                const int r = ntile == 2 ? t : (e & 1);
-                const RingPos<kAS> ar = r ? ar1 : ar0;
+                if (q0 == 0 && !operands(t, x)) goto done;
                 if (nq == 4)
-                  steps(Int<4>{}, q0, r, ar, d, true, f);
+                  steps(Int<4>{}, q0, x, d, true, f, t == G::kH - 1, [] {});
                 else
-                  steps(Int<2>{}, q0, r, ar, d, true, f);
+                  steps(Int<2>{}, q0, x, d, true, f, t == G::kH - 1, [] {});
               }
             }
-            if (ntile == 2 || !(e & 1)) ar0.next();
-            if (ntile == 2 || (e & 1)) ar1.next();
-            xr.next();
+            ar.next();
+            xr.next(G::kH);
           }
         }
         // Rank-r columns: step l of a stage is one branch's 16 columns (A
@@ -663,65 +695,58 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
             const int ls = 4 * (e - KC) + l;
             const bool first = ls == 0 || ls == p.nls_core;
             const bool last = ls == p.nls_core - 1 || ls == p.nls - 1;
-            for (int t = 0; t < ntile; ++t) {
+            for (int t = 0; t < G::kH; ++t) {
+              const RingPos<kXS> x = xr.ahead(t);
               if (first) {
                 uint32_t d, f;
                 if (!acc_start(d, f)) goto done;
                 if (t) d1 = d, f1 = f;
                 else d0 = d, f0 = f;
               }
-              if (l == 0 && !ready_wait(t)) goto done;
+              if (l == 0 && !operands(t, x)) goto done;
               tc_fence_after();
-              const int r = ntile == 2 ? t : (e & 1);
-              const uint32_t slot = r * kAS + (r ? ar1.s : ar0.s);
-              const uint32_t a = tmem_base + G::kABase + slot * 64 + 8 * l;
-              const uint64_t b = xdesc + (uint32_t)(xr.s * (G::kXBytes >> 4)) + (l >> 1) * kBox + 4 * (l & 1);
+              const uint32_t a = tmem_base + G::kABase + ar.s * 64 + 8 * l;
+              const uint32_t ae = a_empty_a + 8 * G::kAParts * ar.s;
+              const uint64_t b = xdesc + (uint32_t)(x.s * (G::kXBytes >> 4)) + (l >> 1) * kBox + 4 * (l & 1);
               const uint32_t d = t ? d1 : d0;
               if (leader) {
                 tc_mma_ts(d, a, b, idesc, !first);
                 tc_mma_ts(d, a, b + 2, idesc, 1);
-                if (l == n - 1) tc_commit_a(a_empty_a + 16 * slot), tc_commit_a(a_empty_a + 16 * slot + 8);
+                if (l == n - 1) {
+                  tc_commit_a(x_empty_a + 8 * x.s);
+                  if (t == G::kH - 1) {
+                    tc_commit_a(ae);
+                    if (G::kAParts == 2) tc_commit_a(ae + 8);
+                  }
+                }
                 if (last) tc_commit_a(t ? f1 : f0);
               }
               __syncwarp();
             }
           }
-          if (ntile == 2 || !(e & 1)) ar0.next();
-          if (ntile == 2 || (e & 1)) ar1.next();
-          xr.next();
+          ar.next();
+          xr.next(G::kH);
         }
       }
     }
-  } else if (warp < 12) {
+  } else if (warp < 4 + 4 * kConv) {
     // ------------------------------ converters ------------------------------
-    // Warpgroup cg converts tile cg of a unit of two tiles, and every other
-    // stage of a unit of one.
-    if constexpr (NT == 128)
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 56;\n" ::: "memory");
-    else
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 64;\n" ::: "memory");
+    // The converter warpgroups take the block's stages in turn, each into its
+    // own A stage.
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(G::kRegsC) : "memory");
     const int cg = (warp - 4) >> 2, cw = warp & 3;
     const int lg = __ffs(p.g) - 1;  // log2 g
-    const uint32_t lane_addr = tmem_base + ((uint32_t)(cw * 32) << 16) + G::kABase + cg * kAS * 64;
-    RingPos<G::kCodeStages> r;
-    RingPos<kXS> xr;
-    RingPos<kAS> ar;
-    // x slots of the last kAS stages this warpgroup converted, newest first
-    // (-1: not its to release): when an A stage is free again, the MMAs that
-    // read it and its x slot are done.  The unit's last tile releases x.
-    int held[kAS];
-#pragma unroll
-    for (int i = 0; i < kAS; ++i) held[i] = -1;
-    for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
-      const int ntile = min(p.tl, p.num_vt - u / p.num_mt * p.tl);
-      const int tile = ntile == 2 ? cg : 0;
-      for (int e = 0; e < KS; ++e) {
-        if (!mbar_wait_warp(&c_full[r.s], r.ph, p.wait_budget, abort_flag, p.err)) goto done;
-        if (ntile == 2 || (e & 1) == cg) {
-          const uint8_t *slot = smem + G::kCodeOff + r.s * G::kCodeSlot;
-          const uint8_t *codes = slot + tile * 2 * kChunkBytes + (cw * 64 + lane) * 16;
-          uint64_t *ae = &a_empty[2 * (cg * kAS + ar.s)];
-          const uint32_t acol = lane_addr + ar.s * 64;
+    const uint32_t acol = tmem_base + ((uint32_t)(cw * 32) << 16) + G::kABase + cg * 64;
+    uint64_t *ae = &a_empty[G::kAParts * cg];
+    RingPos<kCS> cr;
+    cr.next(cg);
+    uint32_t aph = 0;
+    for (int u = blockIdx.x, e = cg;; e += kConv) {
+      while (e >= KS) e -= KS, u += gridDim.x;
+      if (u >= num_units) break;
+      if (!mbar_wait_warp(&c_full[cr.s], cr.ph, p.wait_budget, abort_flag, p.err)) goto done;
+      const uint8_t *slot = smem + G::kCodeOff + cr.s * G::kCodeSlot;
+      const uint8_t *codes = slot + (cw * 64 + lane) * 16;
           if (e < KC) {
             // The warp's codes of the stage first (m-tiles 2 cw and 2 cw + 1 of
             // two 64-wide halves), then the slot is free; one m-tile's
@@ -732,7 +757,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
             uint32_t q[kSC4 ? 4 : 1];  // SC4: scale-code bytes of rows lane/4 + 8 i
             uint32_t q1[kSC4 ? 4 : 1];  // and of the second half where g = 32
             if constexpr (kSC4) {
-              const uint8_t *sb = slot + G::kScaleOff + tile * 2 * kTileRows + cw * 32 + (lane >> 2);
+              const uint8_t *sb = slot + G::kScaleOff + cw * 32 + (lane >> 2);
 #pragma unroll
               for (int i = 0; i < 4; ++i) q[i] = sb[8 * i];
               if (lg == 5) {
@@ -741,7 +766,7 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
               }
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(&c_empty[r.s]);
+            if (lane == 0) mbar_arrive(&c_empty[cr.s]);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const int hf = i >> 1, h = i & 1;
@@ -769,14 +794,14 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
 #pragma unroll
                 for (int k = 0; k < 4; ++k) ah[4 * j + k] = a[k];
               }
-              if (h == 0) {
-                if (!mbar_wait_warp(ae + hf, ar.ph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
+              if (h == 0 && hf < G::kAParts) {
+                if (!mbar_wait_warp(ae + hf, aph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
                 tc_fence_after();
               }
               tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16) + 32 * hf, ah);
             }
           } else {  // four rank-r steps: the first half's 32 columns
-            const uint8_t *lc = slot + tile * 2 * kChunkBytes + (cw * 64 + lane) * 8;
+            const uint8_t *lc = slot + (cw * 64 + lane) * 8;
             const int n = p.nls - 4 * (e - KC);
             uint2 w[8];
 #pragma unroll
@@ -784,8 +809,9 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
               w[i] = i < 4 || n > 2 ? *reinterpret_cast<const uint2 *>(lc + (i >> 1) * kLrStepBytes + (i & 1) * 256)
                                     : make_uint2(0x80808080u, 0x80808080u);
             __syncwarp();
-            if (lane == 0) mbar_arrive(&c_empty[r.s]);
-            if (!mbar_wait_warp(ae + 1, ar.ph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;  // after the first half's
+            if (lane == 0) mbar_arrive(&c_empty[cr.s]);
+            // (The last part's release: the others come before it.)
+            if (!mbar_wait_warp(ae + G::kAParts - 1, aph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
             tc_fence_after();
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -800,55 +826,42 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
               tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16), ah);
             }
           }
-          asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(&ready[tile * kXS + xr.s]);
-            if (cw == 0 && held[kAS - 1] >= 0) mbar_arrive(&x_empty[held[kAS - 1]]);
-          }
-          ar.next();
-#pragma unroll
-          for (int i = kAS - 1; i > 0; --i) held[i] = held[i - 1];
-          held[0] = tile == ntile - 1 ? xr.s : -1;
-        } else {
-          if (lane == 0) mbar_arrive(&c_empty[r.s]);
-        }
-        r.next();
-        xr.next();
-      }
+      asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&a_full[cg]);
+      aph ^= 1;
+      cr.next(kConv);
     }
   } else {
     // ------------------------------ promotion + epilogue ------------------------------
-    if constexpr (NT == 128)
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 160;\n" ::: "memory");
-    else
-      asm volatile("setmaxnreg.inc.sync.aligned.u32 128;\n" ::: "memory");
-    const int tile = (warp - 12) >> 2;  // tile of the unit
-    const int lg = warp & 3;            // TMEM lane group (rows 32*lg .. 32*lg+31)
-    // Cross entropy and greedy read TMEM in the 16x256b shape (4 rows x NT/4
-    // tokens per thread; cross entropy accumulates in base 2, its factors
-    // times log2 e); logits read 32x32b (one row x NT tokens per thread).
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(G::kRegsP) : "memory");
+    const int pw = (warp - 4 - 4 * kConv) >> 2;  // warpgroup: half of the unit's tokens (256), or of the columns (128)
+    const int hf = G::kH == 2 ? pw : 0;
+    const int col0 = TM == 128 ? 64 * pw : 0;    // first accumulator column
+    const int lg = warp & 3;                     // TMEM lane group (rows 32*lg .. 32*lg+31)
+    // Cross entropy and greedy read TMEM in the 16x256b shape (4 rows x
+    // kCols/4 tokens per thread; cross entropy accumulates in base 2, its
+    // factors times log2 e); logits read 32x32b (one row x kCols tokens per thread).
     constexpr bool kQuad = kMode != 0;
     constexpr int kF = kQuad ? 4 : 1;  // rows per thread
     const int rt0 = lg * 32 + (kQuad ? lane >> 2 : lane);
-    const uint32_t lane_addr = tmem_base + ((uint32_t)(lg * 32) << 16);
+    const uint32_t lane_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + col0;
     RingPos<kNB> base;  // the unit's first accumulator
     for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
-      const int vt0 = u / p.num_mt * p.tl;
-      const int ntile = min(p.tl, p.num_vt - vt0);
-      RingPos<kNB> accr = base.ahead(tile);
+      const int64_t vt = u / p.num_mt;
+      const int mu = (u % p.num_mt) * (G::kH * p.nt);
+      RingPos<kNB> accr = base.ahead(hf);
       {
-        const int end = base.s + nb * ntile;
+        const int end = base.s + nb * G::kH;
         base.s = end % kNB;
         base.ph ^= (end / kNB) & 1;
       }
-      if (tile >= ntile) continue;
-      const int64_t vt = vt0 + tile;
-      const int m0 = (u % p.num_mt) * NT;
-      float acc[NT];
+      const int m0 = mu + hf * p.nt + col0;               // token of the thread's first column
+      const int mend = min(p.M, mu + (hf + 1) * p.nt);  // end of the half's tokens
+      float acc[kCols];
 #pragma unroll
-      for (int i = 0; i < NT; ++i) acc[i] = 0.f;
+      for (int i = 0; i < kCols; ++i) acc[i] = 0.f;
       // Promotion factors of a block's rows (rt0, or rt0 + 8k), fp16 bits, loaded a block ahead.
       uint16_t fn[kF];
       const uint16_t *fsrc = (kSC4 ? p.s_row + vt * kTileRows : p.scales + vt * p.G_pad * kTileRows) + rt0;
@@ -875,9 +888,9 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
         tc_fence_after();
         const uint32_t taddr = lane_addr + accr.s * NT;
         // Chunks of 16 registers, the next one loading while one is added.
-        constexpr int kChunks = NT / 16;
-        auto chunk_addr = [&](int c) {  // quad: rows 16 (c / (NT/32)), columns 32 (c % (NT/32))
-          return kQuad ? taddr + ((uint32_t)(16 * (c / (NT / 32))) << 16) + 32 * (c % (NT / 32)) : taddr + 16 * c;
+        constexpr int kChunks = kCols / 16;
+        auto chunk_addr = [&](int c) {  // quad: rows 16 (c / (kCols/32)), columns 32 (c % (kCols/32))
+          return kQuad ? taddr + ((uint32_t)(16 * (c / (kCols / 32))) << 16) + 32 * (c % (kCols / 32)) : taddr + 16 * c;
         };
         uint32_t v[2][16];
         tmem_ld16<kQuad>(chunk_addr(0), v[0]);
@@ -889,40 +902,40 @@ __global__ void __launch_bounds__(kPfThreads, 1) prefill_kernel(const __grid_con
           const uint32_t(&w)[16] = v[c & 1];
 #pragma unroll
           for (int i = 0; i < 16; i += 2) {
-            const float fi = f[kQuad ? 2 * (c / (NT / 32)) + ((i >> 1) & 1) : 0];
+            const float fi = f[kQuad ? 2 * (c / (kCols / 32)) + ((i >> 1) & 1) : 0];
             fma2(a[i], a[i + 1], fi, __uint_as_float(w[i]), __uint_as_float(w[i + 1]));
           }
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[accr.s]);
-        accr.next(ntile);
+        accr.next(G::kH);
       }
       if constexpr (kMode == 0) {
         // Columns are tokens m0 + i, this thread's row is `row`.
         const int64_t row = vt * kTileRows + rt0;
         if (row < p.V) {
-          const int mcount = p.M - m0 < NT ? p.M - m0 : NT;
+          const int mcount = mend - m0 < kCols ? mend - m0 : kCols;
           if (p.out_fp32) {
             float *o = reinterpret_cast<float *>(p.out) + (int64_t)m0 * p.V + row;
 #pragma unroll
-            for (int i = 0; i < NT; ++i, o += p.V)
+            for (int i = 0; i < kCols; ++i, o += p.V)
               if (i < mcount) *o = acc[i];
           } else {
             __nv_bfloat16 *o = reinterpret_cast<__nv_bfloat16 *>(p.out) + (int64_t)m0 * p.V + row;
 #pragma unroll
-            for (int i = 0; i < NT; ++i, o += p.V)
+            for (int i = 0; i < kCols; ++i, o += p.V)
               if (i < mcount) *o = __float2bfloat16_rn(acc[i]);
           }
         }
       } else {
         const int64_t rbase = vt * kTileRows + lg * 32, part = vt * 4 + lg;
         if constexpr (kMode == 2) {
-          quad_argmax<NT, 0>(p, acc, rbase, part, m0, lane);
-          if constexpr (NT == 128) quad_argmax<NT, 1>(p, acc, rbase, part, m0, lane);
+          quad_argmax<kCols, 0>(p, acc, rbase, part, m0, mend, lane);
+          if constexpr (kCols == 128) quad_argmax<kCols, 1>(p, acc, rbase, part, m0, mend, lane);
         } else {
-          quad_ce<NT, 0>(p, acc, rbase, part, m0, lane);
-          if constexpr (NT == 128) quad_ce<NT, 1>(p, acc, rbase, part, m0, lane);
+          quad_ce<kCols, 0>(p, acc, rbase, part, m0, mend, lane);
+          if constexpr (kCols == 128) quad_ce<kCols, 1>(p, acc, rbase, part, m0, mend, lane);
         }
       }
     }
@@ -944,15 +957,15 @@ done:
 // ------------------------------------------------------------------------
 // Host side: tensor maps and launch.
 // ------------------------------------------------------------------------
-template <int NT, int kMode, bool kSC4>
+template <int TM, int kMode, bool kSC4>
 cudaError_t launch_prefill_t(const PrefillParams &p, int grid, bool pdl, cudaStream_t s) {
-  auto kern = prefill_kernel<NT, kMode, kSC4>;
-  cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(kern), PfGeom<NT>::kSmem);
+  auto kern = prefill_kernel<TM, kMode, kSC4>;
+  cudaError_t e = opt_in_smem(reinterpret_cast<const void *>(kern), PfGeom<TM>::kSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(kPfThreads);
-  cfg.dynamicSmemBytes = PfGeom<NT>::kSmem;
+  cfg.blockDim = dim3(PfGeom<TM>::kThreads);
+  cfg.dynamicSmemBytes = PfGeom<TM>::kSmem;
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -968,10 +981,12 @@ cudaError_t launch_prefill_fmt(const archead_pack *pk, const void *x, int M, con
                                int out_fp32, bool argmax, const int32_t *targets, int row0, float2 *ce_part,
                                float *ce_tlogit, bool pdl, cudaStream_t s) {
   PrefillParams p{};
-  // An MMA of up to 128 tokens costs the same whatever its width, so tiles
-  // are 128 tokens; 64 where all tokens fit (smaller x copies, half the
-  // promotion, deeper rings).
-  const int nt = M <= 64 ? 64 : 128;
+  // Conversion of the codes is the same for any number of tokens, so a unit
+  // takes as many as there are, up to 256.
+  const int tm = M <= 64 ? 64 : M <= 128 ? 128 : 256;
+  // Tokens spread evenly over the halves of the units.
+  const int num_mt = (M + tm - 1) / tm, parts = num_mt * (tm == 256 ? 2 : 1);
+  const int nt = ((M + parts - 1) / parts + 15) / 16 * 16;
   if (!make_tma_map_bf16(&p.tmap_x, x, M, pk->d, nt)) return cudaErrorInvalidValue;
   if (pk->lr > 0 && !make_tma_map_bf16(&p.tmap_t, T, M, 2 * pk->lr, nt)) return cudaErrorInvalidValue;
   p.codes = pk->codes;
@@ -983,8 +998,9 @@ cudaError_t launch_prefill_fmt(const archead_pack *pk, const void *x, int M, con
   p.s_a = pk->s_a;
   p.V = pk->V;
   p.M = M;
+  p.nt = nt;
   p.num_vt = pk->num_tiles;
-  p.num_mt = (M + nt - 1) / nt;
+  p.num_mt = num_mt;
   p.d_pad = pk->d_pad;
   p.G_pad = pk->G_pad;
   p.g = pk->g;
@@ -999,24 +1015,17 @@ cudaError_t launch_prefill_fmt(const archead_pack *pk, const void *x, int M, con
   p.ce_tlogit = ce_tlogit;
   p.err = pk->err;
   p.wait_budget = pk->wait_budget;
-  // Two tiles a unit unless one tile a unit leaves the blocks fewer tiles to
-  // do (few units: small heads).
-  const auto rounds = [&](int tl) {
-    const int64_t units = (int64_t)((p.num_vt + tl - 1) / tl) * p.num_mt;
-    return (units + pk->sm_count - 1) / pk->sm_count * tl;
-  };
-  p.tl = 4 * rounds(1) < 3 * rounds(2) ? 1 : 2;
-  const int64_t units = (int64_t)((p.num_vt + p.tl - 1) / p.tl) * p.num_mt;
+  const int64_t units = (int64_t)p.num_vt * p.num_mt;
   if (units > 0x7fffffff - pk->sm_count) return cudaErrorInvalidValue;
   const int grid = (int)(units < pk->sm_count ? units : pk->sm_count);
   const int mode = out ? 0 : argmax ? 2 : 1;
-  if (nt == 64)
-    return mode == 0   ? launch_prefill_t<64, 0, kSC4>(p, grid, pdl, s)
-           : mode == 1 ? launch_prefill_t<64, 1, kSC4>(p, grid, pdl, s)
-                       : launch_prefill_t<64, 2, kSC4>(p, grid, pdl, s);
-  return mode == 0   ? launch_prefill_t<128, 0, kSC4>(p, grid, pdl, s)
-         : mode == 1 ? launch_prefill_t<128, 1, kSC4>(p, grid, pdl, s)
-                     : launch_prefill_t<128, 2, kSC4>(p, grid, pdl, s);
+  const auto run = [&](auto t) {
+    constexpr int TM = decltype(t)::value;
+    return mode == 0   ? launch_prefill_t<TM, 0, kSC4>(p, grid, pdl, s)
+           : mode == 1 ? launch_prefill_t<TM, 1, kSC4>(p, grid, pdl, s)
+                       : launch_prefill_t<TM, 2, kSC4>(p, grid, pdl, s);
+  };
+  return tm == 64 ? run(Int<64>{}) : tm == 128 ? run(Int<128>{}) : run(Int<256>{});
 }
 
 

@@ -144,6 +144,39 @@ def test_logits_many_tokens(name, M):
         gu.check_argmax(got, ref, where=f"{name} M={M} path={path}")
 
 
+# Edges of the tensor-core kernel's instances (64, 128 and 256 tokens a unit),
+# for every group size, ranks that fill, half-fill and skip its rank-r stages,
+# and heads with several vocabulary tiles per block.
+MANY_TILES = {  # more than twice as many tiles as multiprocessors
+    "many_tiles": HeadShape(V=45003, d=320, core_rank=20, corr_rank=12, group_size=64),
+    "sc4_many_tiles": HeadShape(V=45003, d=768, core_rank=10, corr_rank=6, group_size=128, fmt="sc4"),
+}
+EDGE_HEADS = ["g32", "g128", "g256", "core_only", "group_int4", "max_rank", "sc4_ragged", "sc4_g32", "sc4_g256",
+              "many_tiles", "sc4_many_tiles"]
+
+
+@pytest.mark.parametrize("name", EDGE_HEADS)
+@pytest.mark.parametrize("M", [63, 65, 128, 129, 257])
+def test_tensor_core_token_edges(name, M):
+    shape = MANY_TILES.get(name) or SHAPES[name]
+    if name in MANY_TILES and name not in _packs:
+        head = make_head(shape, seed=5)
+        _packs[name] = (archead.archead_pack_create(head, shape), head)
+    pack, head = get(name)
+    x = make_hidden(shape.d, M, seed=700 + M)
+    ref = oracle.logits(head, shape, x)
+    got = gu.forward(pack, x, archead.OUT_FP32, archead.PATH_PREFILL)
+    gu.check_logits(got, ref, where=f"{name} M={M}")
+    idx, val = gu.forward_argmax(pack, x, archead.PATH_PREFILL)
+    gu.check_greedy(idx, val, ref, where=f"{name} M={M}")
+    t = make_targets(shape.V, M, seed=M)
+    ce, st = gu.forward_ce(pack, x, t, archead.PATH_PREFILL)
+    assert st == archead.OK
+    mx = ref.max(axis=1)
+    lse = mx + np.log(np.exp(ref - mx[:, None]).sum(axis=1))
+    assert np.max(np.abs(ce - (lse - ref[np.arange(M), t]))) <= gu.CE_ABS
+
+
 @pytest.mark.parametrize("name", ["ragged", "tiny", "g32", "g256", "corr_only", "one_row", "max_rank", "sc4",
                                   "sc4_g32"])
 @pytest.mark.parametrize("M", [1, 7, 16, 40])
