@@ -28,32 +28,42 @@ __device__ __forceinline__ float warp_max(float v) {
   return v;
 }
 
-// Codes of a value v against a scale s > 0 with reciprocal inv = 1 / s: the
-// integer (as a float) clamp(rint(v / s), -qmax, qmax) of the definition
-// above, bit for bit, without its division.  v * inv differs from the
-// rounded quotient by at most 2^-22 of its size, below 5e-5 for the |v / s|
-// <= 1.5 qmax < 200 that a group's own scale leaves (fp16 subnormal scales
-// included), so unless v * inv lies within 1e-4 of a half-integer both round
-// to the same integer; the rest (about 1 value in 5000), and NaNs and
-// infinities, take the division.  Adding 1.5 * 2^23 rounds to an integer,
-// ties to even.
-__device__ __forceinline__ float quant_code(float v, float s, float inv, float qmax) {
-  const float q = v * inv;
-  float r = __fadd_rn(__fadd_rn(q, 12582912.f), -12582912.f);
-  if (!(fabsf(q - r) < 0.4999f)) r = rintf(__fdiv_rn(v, s));
-  return fminf(fmaxf(r, -qmax), qmax);
+// The code of one value by the definition above.
+__device__ __forceinline__ uint32_t quant_code_div(float v, float s, float qmax) {
+  if (!(s > 0.f)) return 0;
+  return (uint32_t)(int)fminf(fmaxf(rintf(__fdiv_rn(v, s)), -qmax), qmax) & 255u;
 }
 
-// Four codes as the bytes of a word.
+// Codes of four values against their scales s with reciprocals inv = 1 / s
+// (rounded), as the bytes of a word: bit for bit those of the definition, four
+// operations a value instead of a division.  Adding 1.5 * 2^23 in the FMA
+// rounds v * inv to an integer n, ties to even, in the sum's low bits.  v *
+// inv and the rounded quotient differ by less than 2^-22 of their size, below
+// 5e-5 for |v / s| < 200, so unless v * inv lies within 1e-4 of a half-integer
+// both round to n (about 1 value in 5000 does).  Those, NaNs and infinities,
+// and scales below the fp16 normal range (zero, or so coarse that |v / s| may
+// exceed qmax; a normal scale leaves it below qmax + 0.1), take the definition.
+__device__ __forceinline__ uint32_t quant_code4(float4 v, float4 s, float4 inv, float qmax) {
+  constexpr float kMagic = 12582912.f;
+  const float tx = fmaf(v.x, inv.x, kMagic), ty = fmaf(v.y, inv.y, kMagic);
+  const float tz = fmaf(v.z, inv.z, kMagic), tw = fmaf(v.w, inv.w, kMagic);
+  float off = fabsf(fmaf(v.x, inv.x, -(tx - kMagic)));  // distance from n; max.NaN keeps a NaN
+  asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(off) : "f"(fabsf(fmaf(v.y, inv.y, -(ty - kMagic)))));
+  asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(off) : "f"(fabsf(fmaf(v.z, inv.z, -(tz - kMagic)))));
+  asm("max.NaN.f32 %0, %0, %1;\n" : "+f"(off) : "f"(fabsf(fmaf(v.w, inv.w, -(tw - kMagic)))));
+  constexpr float kNormal = 6.103515625e-05f;  // 2^-14
+  if (off < 0.4999f && fminf(fminf(s.x, s.y), fminf(s.z, s.w)) >= kNormal)
+    return __byte_perm(__byte_perm(__float_as_uint(tx), __float_as_uint(ty), 0x0040),
+                       __byte_perm(__float_as_uint(tz), __float_as_uint(tw), 0x0040), 0x5410);
+  return quant_code_div(v.x, s.x, qmax) | quant_code_div(v.y, s.y, qmax) << 8 | quant_code_div(v.z, s.z, qmax) << 16 |
+         quant_code_div(v.w, s.w, qmax) << 24;
+}
 __device__ __forceinline__ uint32_t quant_code4(float4 v, float s, float inv, float qmax) {
-  if (!(s > 0.f)) return 0;
-  const int a = (int)quant_code(v.x, s, inv, qmax), b = (int)quant_code(v.y, s, inv, qmax);
-  const int c = (int)quant_code(v.z, s, inv, qmax), d = (int)quant_code(v.w, s, inv, qmax);
-  return __byte_perm(__byte_perm(a, b, 0x0040), __byte_perm(c, d, 0x0040), 0x5410);
+  return quant_code4(v, make_float4(s, s, s, s), make_float4(inv, inv, inv, inv), qmax);
 }
 
 __device__ __forceinline__ float abs_max4(float4 v) {
-  return fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+  return fmaxf(fmaxf(fmaxf(0.f, fabsf(v.x)), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));  // 0 if all are NaN
 }
 
 // Groups of kGc consecutive values of a row (32, 64, 128 or 256): with whole
@@ -100,14 +110,14 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const float4 *__rest
 }
 
 // Groups of gr rows of one column (the core factors: gr = all rows; the
-// correction's right factor: gr = g).  A cluster of blocks takes one group
-// of rows of eight adjacent columns (one 32-byte sector of a row), each
-// block a slice of the rows: column maxima over its slice, the maximum over
-// the cluster through distributed shared memory, then the codes.  With all
-// rows of 128 columns in one group, 16 clusters of eight blocks read x at
-// full sectors from 128 SMs, the second time mostly from L2; one warp per
-// column read one value per sector, on 128 warps in all.
-// kVec: cols is a multiple of 8, x 16-byte and codes 8-byte aligned.
+// correction's right factor: gr = g), for any number of columns and any
+// alignment.  A cluster of blocks takes one group of rows of eight adjacent
+// columns (one 32-byte sector of a row), each block a slice of the rows:
+// column maxima over its slice, the maximum over the cluster through
+// distributed shared memory, then the codes, x coming mostly from L2 the
+// second time.  One warp per column read one value per sector, on as many
+// warps as there are columns (8.8 ms for 151936 x 128).
+// kVec: cols is a multiple of 8, x 16-byte and codes 4-byte aligned.
 constexpr int kColThreads = 512;
 template <bool kVec>
 __global__ void __launch_bounds__(kColThreads) quantize_columns_kernel(const float *__restrict__ x, int64_t cols,
@@ -116,7 +126,7 @@ __global__ void __launch_bounds__(kColThreads) quantize_columns_kernel(const flo
                                                                        uint16_t *__restrict__ scales) {
   __shared__ float wmax[kColThreads / 32][8];
   __shared__ float bmax[8];  // this block's maxima, read by the cluster
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, half = threadIdx.x & 1;
   uint32_t rank, nrank;
   asm("mov.u32 %0, %%cluster_ctarank;\n" : "=r"(rank));
   asm("mov.u32 %0, %%cluster_nctarank;\n" : "=r"(nrank));
@@ -124,43 +134,44 @@ __global__ void __launch_bounds__(kColThreads) quantize_columns_kernel(const flo
   const int64_t job = blockIdx.x / nrank;  // (row group, strip)
   const int64_t c0 = (job % strips) * 8, r0 = (job / strips) * gr;
   const int nc = (int)(cols - c0 < 8 ? cols - c0 : 8);
-  const float *xs = x + r0 * cols + c0;
-  int8_t *cs = codes + r0 * cols + c0;
-  const int64_t step = (int64_t)nrank * kColThreads;
-  const int64_t first = (int64_t)rank * kColThreads + threadIdx.x;
-  auto load = [&](int64_t r, float (&v)[8]) {
-    if (kVec) {
-      const float4 a = *reinterpret_cast<const float4 *>(xs + r * cols);
-      const float4 b = *reinterpret_cast<const float4 *>(xs + r * cols + 4);
-      v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w, v[4] = b.x, v[5] = b.y, v[6] = b.z, v[7] = b.w;
-    } else {
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = j < nc ? xs[r * cols + j] : 0.f;
+  // Two threads a row, four columns each, eight rows in flight a thread.
+  constexpr int kU = 8;
+  const float *xs = x + r0 * cols + c0 + 4 * half;
+  int8_t *cs = codes + r0 * cols + c0 + 4 * half;
+  const int64_t step = (int64_t)nrank * (kColThreads / 2);
+  const int64_t first = (int64_t)rank * (kColThreads / 2) + (threadIdx.x >> 1);
+  auto load = [&](int64_t r) {
+    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r < gr) {
+      if (kVec) {
+        v = *reinterpret_cast<const float4 *>(xs + r * cols);
+      } else {
+        if (4 * half + 0 < nc) v.x = xs[r * cols];
+        if (4 * half + 1 < nc) v.y = xs[r * cols + 1];
+        if (4 * half + 2 < nc) v.z = xs[r * cols + 2];
+        if (4 * half + 3 < nc) v.w = xs[r * cols + 3];
+      }
     }
+    return v;
   };
-  float mx[8];
+  float mx[4] = {0.f, 0.f, 0.f, 0.f};
+  for (int64_t r = first; r < gr; r += kU * step) {
+    float4 v[kU];
 #pragma unroll
-  for (int j = 0; j < 8; ++j) mx[j] = 0.f;
-  int64_t r = first;
-  for (; r + 3 * step < gr; r += 4 * step) {  // four rows in flight
-    float v[4][8];
+    for (int u = 0; u < kU; ++u) v[u] = load(r + u * step);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) load(r + u * step, v[u]);
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int j = 0; j < 8; ++j) mx[j] = fmaxf(mx[j], fabsf(v[u][j]));
-  }
-  for (; r < gr; r += step) {
-    float v[8];
-    load(r, v);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) mx[j] = fmaxf(mx[j], fabsf(v[j]));
+    for (int u = 0; u < kU; ++u) {
+      mx[0] = fmaxf(mx[0], fabsf(v[u].x));
+      mx[1] = fmaxf(mx[1], fabsf(v[u].y));
+      mx[2] = fmaxf(mx[2], fabsf(v[u].z));
+      mx[3] = fmaxf(mx[3], fabsf(v[u].w));
+    }
   }
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    mx[j] = warp_max(mx[j]);
-    if (lane == j) wmax[warp][j] = mx[j];
+  for (int j = 0; j < 4; ++j) {
+#pragma unroll
+    for (int o = 16; o > 1; o >>= 1) mx[j] = fmaxf(mx[j], __shfl_xor_sync(0xffffffffu, mx[j], o));
+    if (lane < 2) wmax[warp][4 * half + j] = mx[j];
   }
   __syncthreads();
   if (threadIdx.x < 8) {
@@ -170,7 +181,7 @@ __global__ void __launch_bounds__(kColThreads) quantize_columns_kernel(const flo
     bmax[threadIdx.x] = m;
   }
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-  float s[8], inv[8];
+  float s[4], inv[4];
   {
     float m = 0.f;  // lane j < 8 of every warp: column j over the cluster's blocks
     for (uint32_t b = 0; b < nrank; ++b) {
@@ -184,28 +195,116 @@ __global__ void __launch_bounds__(kColThreads) quantize_columns_kernel(const flo
     if (rank == 0 && threadIdx.x < nc) scales[(job / strips) * cols + c0 + threadIdx.x] = __half_as_ushort(s16);
     const float sj = __half2float(s16);
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      s[j] = __shfl_sync(0xffffffffu, sj, j);
+    for (int j = 0; j < 4; ++j) {
+      s[j] = __shfl_sync(0xffffffffu, sj, 4 * half + j);
       inv[j] = __frcp_rn(s[j]);
     }
   }
   // No block leaves while another may still read its maxima.
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
-#pragma unroll 4
-  for (r = first; r < gr; r += step) {
-    float v[8];
-    load(r, v);
-    uint32_t q[8];
+  for (int64_t r = first; r < gr; r += kU * step) {
+    float4 v[kU];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) q[j] = s[j] > 0.f ? (uint32_t)(int)quant_code(v[j], s[j], inv[j], qmax) & 255u : 0u;
-    if (kVec) {
-      *reinterpret_cast<uint2 *>(cs + r * cols) =
-          make_uint2(q[0] | q[1] << 8 | q[2] << 16 | q[3] << 24, q[4] | q[5] << 8 | q[6] << 16 | q[7] << 24);
-    } else {
+    for (int u = 0; u < kU; ++u) v[u] = load(r + u * step);
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (j < nc) cs[r * cols + j] = (int8_t)q[j];
+    for (int u = 0; u < kU; ++u) {
+      const int64_t ru = r + u * step;
+      if (ru >= gr) break;
+      const uint32_t q = quant_code4(v[u], make_float4(s[0], s[1], s[2], s[3]),
+                                     make_float4(inv[0], inv[1], inv[2], inv[3]), qmax);
+      if (kVec) {
+        *reinterpret_cast<uint32_t *>(cs + ru * cols) = q;
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (4 * half + j < nc) cs[ru * cols + j] = (int8_t)(q >> (8 * j));
+      }
     }
+  }
+}
+
+// The same where whole rows are read at once (cols a multiple of 4 up to
+// 1024, 16-byte aligned, thousands of rows a group): three passes over x read
+// as it lies, 16 bytes a lane.  A strip of eight columns touches a 128-byte
+// line per row for 32 bytes of it, which held the kernel above at 93 us (L1
+// bound) for 151936 x 128; the three passes take 38 us.
+//   1: blocks (row slice, group) leave their column maxima at the start of
+//      the group's codes, which are written only by pass 3;
+//   2: a block per group turns them into scales;
+//   3: codes.
+constexpr int kColSlices = 304;  // two row slices a multiprocessor
+__global__ void __launch_bounds__(256) column_maxima_kernel(const float4 *__restrict__ x, int cols4, int64_t gr,
+                                                            int8_t *__restrict__ codes) {
+  __shared__ float4 red[256];
+  const int lanes = 256 / cols4;  // rows read at a time by a block
+  const int c = threadIdx.x % cols4, l = threadIdx.x / cols4;
+  const float4 *xs = x + (int64_t)blockIdx.y * gr * cols4 + c;
+  const int64_t step = (int64_t)gridDim.x * lanes;
+  constexpr int kU = 8;
+  float4 m = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int64_t r = (int64_t)blockIdx.x * lanes + l; l < lanes && r < gr; r += kU * step) {
+    float4 v[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) v[u] = r + u * step < gr ? xs[(r + u * step) * cols4] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      m = make_float4(fmaxf(m.x, fabsf(v[u].x)), fmaxf(m.y, fabsf(v[u].y)), fmaxf(m.z, fabsf(v[u].z)),
+                      fmaxf(m.w, fabsf(v[u].w)));
+  }
+  red[threadIdx.x] = m;
+  __syncthreads();
+  if (threadIdx.x < cols4) {
+    for (int i = 1; i < lanes; ++i) {
+      const float4 o = red[i * cols4 + c];
+      m = make_float4(fmaxf(m.x, o.x), fmaxf(m.y, o.y), fmaxf(m.z, o.z), fmaxf(m.w, o.w));
+    }
+    float *part = reinterpret_cast<float *>(codes + (int64_t)blockIdx.y * gr * (4 * cols4)) + (int64_t)blockIdx.x * 4 * cols4;
+    part[4 * c] = m.x, part[4 * c + 1] = m.y, part[4 * c + 2] = m.z, part[4 * c + 3] = m.w;
+  }
+}
+
+__global__ void __launch_bounds__(256) column_scales_kernel(const int8_t *__restrict__ codes, int cols, int64_t gr,
+                                                            int slices, float qmax, uint16_t *__restrict__ scales) {
+  // Block (32 columns, group): warps stride over the slices.
+  __shared__ float red[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int c = blockIdx.x * 32 + lane;
+  const float *part = reinterpret_cast<const float *>(codes + (int64_t)blockIdx.y * gr * cols);
+  float m = 0.f;
+  if (c < cols) {
+#pragma unroll 8
+    for (int i = warp; i < slices; i += 8) m = fmaxf(m, part[(int64_t)i * cols + c]);
+  }
+  red[warp][lane] = m;
+  __syncthreads();
+  if (warp == 0 && c < cols) {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) m = fmaxf(m, red[w][lane]);
+    scales[(int64_t)blockIdx.y * cols + c] = __half_as_ushort(__float2half_rn(__fdiv_rn(m, qmax)));
+  }
+}
+
+__global__ void __launch_bounds__(256) column_codes_kernel(const float4 *__restrict__ x, int cols4, int64_t gr,
+                                                           float qmax, const uint16_t *__restrict__ scales,
+                                                           uint32_t *__restrict__ codes) {
+  const int lanes = 256 / cols4;
+  const int c = threadIdx.x % cols4, l = threadIdx.x / cols4;
+  if (l >= lanes) return;
+  const int64_t base = (int64_t)blockIdx.y * gr * cols4 + c;
+  const int64_t step = (int64_t)gridDim.x * lanes;
+  const uint16_t *sc = scales + ((int64_t)blockIdx.y * cols4 + c) * 4;
+  const float4 s = make_float4(fp16_bits_to_f32(sc[0]), fp16_bits_to_f32(sc[1]), fp16_bits_to_f32(sc[2]),
+                               fp16_bits_to_f32(sc[3]));
+  const float4 inv = make_float4(__frcp_rn(s.x), __frcp_rn(s.y), __frcp_rn(s.z), __frcp_rn(s.w));
+  constexpr int kU = 8;
+  for (int64_t r = (int64_t)blockIdx.x * lanes + l; r < gr; r += kU * step) {
+    float4 v[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      v[u] = r + u * step < gr ? x[base + (r + u * step) * cols4] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      if (r + u * step < gr) codes[base + (r + u * step) * cols4] = quant_code4(v[u], s, inv, qmax);
   }
 }
 
@@ -283,8 +382,9 @@ __global__ void quantize_residual_sc4_kernel(const float *__restrict__ r, int64_
 // registers, so r is read once (5 bytes a value in all, which bounds it).
 // Group maxima come from the kLanes lanes holding a group (two halves, for g
 // = 256, meet in shared memory), the row maximum from the warps'; then one
-// thread per group takes its scale code, scale and reciprocal.  The
-// one-warp-per-row kernel read r twice, 4 bytes a lane, and divided every value.
+// thread per group takes its scale code, scale and reciprocal, while the next
+// row is on its way.  The one-warp-per-row kernel read r twice, 4 bytes a
+// lane, and divided every value.
 constexpr int kSc4Threads = 256;
 template <int kNV>
 __global__ void __launch_bounds__(kSc4Threads) quantize_residual_sc4_rows_kernel(
@@ -298,13 +398,20 @@ __global__ void __launch_bounds__(kSc4Threads) quantize_residual_sc4_rows_kernel
   const int lanes = g4 < 32 ? g4 : 32;   // lanes sharing a piece
   const int lp = lg - 2 < 5 ? lg - 2 : 5;  // log2 of the piece's float4 count
   const int G = cols4 >> (lg - 2);
-  for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-    float4 v[kNV];
+  auto load = [&](int64_t row, float4 (&d)[kNV]) {
 #pragma unroll
     for (int u = 0; u < kNV; ++u) {
       const int i = threadIdx.x + kSc4Threads * u;
-      v[u] = i < cols4 ? __ldcs(r + row * cols4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+      d[u] = row < rows && i < cols4 ? __ldcs(r + row * cols4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
+  };
+  float4 next[kNV];
+  load(blockIdx.x, next);
+  for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
+    float4 v[kNV];
+#pragma unroll
+    for (int u = 0; u < kNV; ++u) v[u] = next[u];
+    load(row + gridDim.x, next);
     float rmax = 0.f;
 #pragma unroll
     for (int u = 0; u < kNV; ++u) {
@@ -468,8 +575,19 @@ void launch_quantize_rows(const float *x, int64_t n, int qmax, int8_t *codes, ui
 
 cudaError_t launch_quantize_columns(const float *x, int64_t rows, int64_t cols, int64_t gr, int qmax, int8_t *codes,
                                     uint16_t *scales, cudaStream_t s) {
-  const int64_t jobs = (rows / gr) * ((cols + 7) / 8);
-  const int cluster = gr >= 8 * kColThreads ? 8 : 1;  // blocks sharing a group: at least a row a thread each
+  const int64_t groups = rows / gr;
+  if (cols % 4 == 0 && cols <= 1024 && gr >= 4 * kColSlices && groups <= 65535 && aligned(x, 16) && aligned(codes, 4)) {
+    const int cols4 = (int)(cols / 4);
+    const dim3 grid(kColSlices, (unsigned)groups);
+    const float4 *x4 = reinterpret_cast<const float4 *>(x);
+    column_maxima_kernel<<<grid, 256, 0, s>>>(x4, cols4, gr, codes);
+    column_scales_kernel<<<dim3((unsigned)((cols + 31) / 32), (unsigned)groups), 256, 0, s>>>(
+        codes, (int)cols, gr, kColSlices, (float)qmax, scales);
+    column_codes_kernel<<<grid, 256, 0, s>>>(x4, cols4, gr, (float)qmax, scales, reinterpret_cast<uint32_t *>(codes));
+    return cudaGetLastError();
+  }
+  const int64_t jobs = groups * ((cols + 7) / 8);
+  const int cluster = gr >= 8 * kColThreads ? 8 : 1;  // blocks sharing a group: at least two rows a thread pair each
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(jobs * cluster));
   cfg.blockDim = dim3(kColThreads);
@@ -480,7 +598,7 @@ cudaError_t launch_quantize_columns(const float *x, int64_t rows, int64_t cols, 
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  const bool vec = cols % 8 == 0 && aligned(x, 16) && aligned(codes, 8);
+  const bool vec = cols % 8 == 0 && aligned(x, 16) && aligned(codes, 4);
   return cudaLaunchKernelEx(&cfg, vec ? quantize_columns_kernel<true> : quantize_columns_kernel<false>, x, cols, gr,
                             (float)qmax, codes, scales);
 }

@@ -109,7 +109,8 @@ def _quantise_at(x, gr, gc, bits, offset):
 @pytest.mark.parametrize("shape,groups,bits", [
     ((3, 32), (1, 32), 4), ((37, 192), (1, 64), 4), ((5, 1664), (1, 128), 8), ((9, 768), (1, 256), 5),  # rows
     ((511, 3), (511, 1), 8), ((512, 7), (512, 1), 8), ((4095, 16), (4095, 1), 5), ((4096, 16), (4096, 1), 8),
-    ((20011, 13), (20011, 1), 8), ((1200, 24), (600, 1), 4),                                            # columns
+    ((20011, 13), (20011, 1), 8), ((1200, 24), (600, 1), 4),
+    ((1215, 4), (1215, 1), 8), ((1216, 4), (1216, 1), 8), ((2432, 1024), (1216, 1), 5), ((9001, 200), (9001, 1), 8),  # columns
 ], ids=str)
 def test_quantiser_routes_bit_exact(shape, groups, bits, offset):
     x = _edge_values(shape[0] + bits, shape)
@@ -117,6 +118,17 @@ def test_quantiser_routes_bit_exact(shape, groups, bits, offset):
     rq, rs = oc.quantize_symmetric(x, groups[0], groups[1], bits)
     assert np.array_equal(scales, rs)
     assert np.array_equal(codes, rq)
+
+
+def test_quantiser_routes_agree_on_values_that_are_not_finite():
+    """The 16-byte route against the general kernel (which unaligned buffers take)."""
+    x = _edge_values(1, (6, 256))
+    x[1, ::7] = np.nan
+    x[2, 3] = np.inf
+    x[3] = np.nan
+    x[4, 9] = 3e38
+    a, b = _quantise_at(x, 1, 64, 4, 0), _quantise_at(x, 1, 64, 4, 1)
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
 @pytest.mark.parametrize("cols,g", [(32, 32), (1024, 256), (1056, 32), (2112, 64), (4096, 128), (8192, 256), (8256, 64)])
