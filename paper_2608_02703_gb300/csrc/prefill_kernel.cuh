@@ -36,19 +36,20 @@
 // 128 bytes a cycle that shared memory moves, and it ran at 62 % of the
 // measured tensor peak.  With A in TMEM an MMA of N tokens takes about N / 2 +
 // 5 cycles (measured alone: 39 for 64, 67 for 128), and what is left is the
-// issuing warp's own instructions (two turns a stage: about 1350 cycles, 1070
+// issuing warp's own instructions (two turns a stage: about 1400 cycles, 1070
 // of them MMAs) and, below 129 tokens, the conversion of the codes, which does
-// not depend on the tokens.  Qwen3-8B shape, start and now: 24 tokens 150 ->
-// 142 us, 64 tokens 246 -> 149, 4096 tokens 4.47 -> 3.72 ms; the paper's
-// format 200 tokens 319 -> 220 us, cross entropy of 2048 tokens 2.14 -> 1.72
-// ms; Gemma shape, cross entropy of 512 tokens 781 -> 684 us.
+// not depend on the tokens.  Qwen3-8B shape, before and now: 24 tokens 150 ->
+// 137 us, 64 tokens 246 -> 143, 4096 tokens 4.51 -> 3.66 ms; the paper's
+// format 200 tokens 318 -> 222 us, cross entropy of 2048 tokens 2.15 -> 1.74
+// ms; Gemma shape, cross entropy of 512 tokens 776 -> 667 us.
 //
 // Epilogues: logits (each promotion thread stores one row of its tokens),
 // greedy partials (largest logit and its row per token over each warp's 32
 // rows) and cross-entropy partials (max and sum of exp per token over each
-// warp's 32 rows, plus the target's logit).  The cross-entropy and greedy
-// instances read TMEM in the 16x256b shape, so that a thread holds 4 rows
-// of a quarter of them and most of the reduction over rows is thread-local.
+// warp's 32 rows, plus the target's logit).  For the latter two a unit's sums
+// pass through TMEM once more, read back in the 16x256b shape, so that a
+// thread holds 4 rows of a quarter of the tokens and most of the reduction
+// over rows is thread-local.
 #pragma once
 
 #include <cfloat>
@@ -173,6 +174,24 @@ __device__ __forceinline__ void tmem_st_frag4(uint32_t taddr, const uint32_t (&a
           taddr),
       "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(a[4]), "r"(a[5]), "r"(a[6]), "r"(a[7]), "r"(a[8]), "r"(a[9]),
       "r"(a[10]), "r"(a[11]), "r"(a[12]), "r"(a[13]), "r"(a[14]), "r"(a[15])
+      : "memory");
+}
+
+// 32 lanes x 32 columns from registers, one value per column per thread.
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float *a) {
+  asm volatile(
+      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,"
+      "%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};\n" ::"r"(taddr),
+      "r"(__float_as_uint(a[0])), "r"(__float_as_uint(a[1])), "r"(__float_as_uint(a[2])), "r"(__float_as_uint(a[3])),
+      "r"(__float_as_uint(a[4])), "r"(__float_as_uint(a[5])), "r"(__float_as_uint(a[6])), "r"(__float_as_uint(a[7])),
+      "r"(__float_as_uint(a[8])), "r"(__float_as_uint(a[9])), "r"(__float_as_uint(a[10])),
+      "r"(__float_as_uint(a[11])), "r"(__float_as_uint(a[12])), "r"(__float_as_uint(a[13])),
+      "r"(__float_as_uint(a[14])), "r"(__float_as_uint(a[15])), "r"(__float_as_uint(a[16])),
+      "r"(__float_as_uint(a[17])), "r"(__float_as_uint(a[18])), "r"(__float_as_uint(a[19])),
+      "r"(__float_as_uint(a[20])), "r"(__float_as_uint(a[21])), "r"(__float_as_uint(a[22])),
+      "r"(__float_as_uint(a[23])), "r"(__float_as_uint(a[24])), "r"(__float_as_uint(a[25])),
+      "r"(__float_as_uint(a[26])), "r"(__float_as_uint(a[27])), "r"(__float_as_uint(a[28])),
+      "r"(__float_as_uint(a[29])), "r"(__float_as_uint(a[30])), "r"(__float_as_uint(a[31]))
       : "memory");
 }
 
@@ -875,12 +894,13 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
     const int hf = G::kH == 2 ? pw : 0;
     const int col0 = TM == 128 ? 64 * pw : 0;    // first accumulator column
     const int lg = warp & 3;                     // TMEM lane group (rows 32*lg .. 32*lg+31)
-    // Cross entropy and greedy read TMEM in the 16x256b shape (4 rows x
-    // kCols/4 tokens per thread; cross entropy accumulates in base 2, its
-    // factors times log2 e); logits read 32x32b (one row x kCols tokens per thread).
-    constexpr bool kQuad = kMode != 0;
-    constexpr int kF = kQuad ? 4 : 1;  // rows per thread
-    const int rt0 = lg * 32 + (kQuad ? lane >> 2 : lane);
+    // A thread sums one row x kCols tokens (32x32b).  Cross entropy and greedy
+    // reduce over rows, with 4 rows x kCols/4 tokens per thread (16x256b): their
+    // sums change shape through the tensor memory of the unit's last block.
+    // (Promoting in that shape takes four factors a thread and half-height
+    // loads for every block: 4.27 against 3.35 ms for 4096 tokens, Qwen3-8B
+    // shape.)  Cross entropy accumulates in base 2, its factors times log2 e.
+    const int rt0 = lg * 32 + lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + col0;
     RingPos<kNB> base;  // the unit's first accumulator
     for (int u = blockIdx.x; u < num_units; u += gridDim.x) {
@@ -897,48 +917,48 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
       float acc[kCols];
 #pragma unroll
       for (int i = 0; i < kCols; ++i) acc[i] = 0.f;
-      // Promotion factors of a block's rows (rt0, or rt0 + 8k), fp16 bits, loaded a block ahead.
-      uint16_t fn[kF];
+      // Promotion factor of a block's row, fp16 bits, loaded a block ahead.
       const uint16_t *fsrc = (kSC4 ? p.s_row + vt * kTileRows : p.scales + vt * p.G_pad * kTileRows) + rt0;
-#pragma unroll
-      for (int k = 0; k < kF; ++k) fn[k] = fsrc[8 * k];
+      uint16_t fn = *fsrc;
       for (int b = 0; b < nb; ++b) {
-        float f[kF];
-#pragma unroll
-        for (int k = 0; k < kF; ++k) f[k] = fp16_bits_to_f32(fn[k]) * (kMode == 1 ? kLog2e : 1.f);
+        const float f = fp16_bits_to_f32(fn) * (kMode == 1 ? kLog2e : 1.f);
         if (b + 1 < nres) {
           if (!kSC4) {
             fsrc += kTileRows;
-#pragma unroll
-            for (int k = 0; k < kF; ++k) fn[k] = fsrc[8 * k];
+            fn = *fsrc;
           }
         } else if (b + 1 == nres && has_core) {
-#pragma unroll
-          for (int k = 0; k < kF; ++k) fn[k] = 0x3C00;  // 1
+          fn = 0x3C00;  // 1
         } else if (has_corr) {
-#pragma unroll
-          for (int k = 0; k < kF; ++k) fn[k] = p.s_a[vt * kTileRows + rt0 + 8 * k];
+          fn = p.s_a[vt * kTileRows + rt0];
         }
         if (!mbar_wait_warp(&acc_full[accr.s], accr.ph, p.wait_budget, abort_flag, p.err)) goto done;
         tc_fence_after();
         const uint32_t taddr = lane_addr + accr.s * NT;
         // Chunks of 16 registers, the next one loading while one is added.
         constexpr int kChunks = kCols / 16;
-        auto chunk_addr = [&](int c) {  // quad: rows 16 (c / (kCols/32)), columns 32 (c % (kCols/32))
-          return kQuad ? taddr + ((uint32_t)(16 * (c / (kCols / 32))) << 16) + 32 * (c % (kCols / 32)) : taddr + 16 * c;
-        };
         uint32_t v[2][16];
-        tmem_ld16<kQuad>(chunk_addr(0), v[0]);
+        tmem_ld16<false>(taddr, v[0]);
 #pragma unroll
         for (int c = 0; c < kChunks; ++c) {
           tmem_wait_ld(v[c & 1]);
-          if (c + 1 < kChunks) tmem_ld16<kQuad>(chunk_addr(c + 1), v[(c + 1) & 1]);
+          if (c + 1 < kChunks) tmem_ld16<false>(taddr + 16 * (c + 1), v[(c + 1) & 1]);
           float *a = acc + 16 * c;
           const uint32_t(&w)[16] = v[c & 1];
 #pragma unroll
-          for (int i = 0; i < 16; i += 2) {
-            const float fi = f[kQuad ? 2 * (c / (kCols / 32)) + ((i >> 1) & 1) : 0];
-            fma2(a[i], a[i + 1], fi, __uint_as_float(w[i]), __uint_as_float(w[i + 1]));
+          for (int i = 0; i < 16; i += 2) fma2(a[i], a[i + 1], f, __uint_as_float(w[i]), __uint_as_float(w[i + 1]));
+        }
+        if (kMode != 0 && b + 1 == nb) {
+          // To the shape of the row reductions, through the drained block.
+#pragma unroll
+          for (int c = 0; c < kCols; c += 32) tmem_st32(taddr + c, acc + c);
+          asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+#pragma unroll
+          for (int c = 0; c < kChunks; ++c) {  // rows 16 (c / (kCols/32)), columns 32 (c % (kCols/32))
+            tmem_ld16<true>(taddr + ((uint32_t)(16 * (c / (kCols / 32))) << 16) + 32 * (c % (kCols / 32)), v[0]);
+            tmem_wait_ld(v[0]);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) acc[16 * c + i] = __uint_as_float(v[0][i]);
           }
         }
         tc_fence_before();
