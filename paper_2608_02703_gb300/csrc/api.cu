@@ -224,12 +224,18 @@ archead_status run_prefill(archead_pack *p, const void *x, int64_t M, void *out,
   // Few tokens: the pre-pass that splits d over blocks (the tensor-core one
   // runs M / 64 blocks per 32 columns, each over the whole of d).
   const bool split_pre = M <= kPrefillSplitPrepass;
-  size_t partial_off = 0;
+  size_t partial_off = 0, reserve = 0;
   if (split_pre) {
     partial_off = c.take(prepass_partial_bytes((int)M, p->lr, p->d));
     AH_CUDA(ensure_counters(p, prepass_pairs((int)M, p->lr), s));
+  } else {
+    // A call with more tokens leaves room for any with fewer, partial sums
+    // included, so that those need no growth (under stream capture, say).
+    reserve = (size_t)kPrefillSplitPrepass * std::max(2 * p->lr, 64) * 2 + 256 +
+              prepass_partial_bytes(kPrefillSplitPrepass, p->lr, p->d);
+    if (ce_mode) reserve += (size_t)kPrefillSplitPrepass * (p->num_tiles * prefill_parts_per_vt() * sizeof(float2) + 4) + 512;
   }
-  AH_CUDA(ensure_workspace(p, c.off, s));
+  AH_CUDA(ensure_workspace(p, std::max(c.off, reserve), s));
   PrepassParams pp = prepass_params(p, x, M);
   pp.ts = nullptr;
   pp.T = at<uint16_t>(p->ws, t_off);
@@ -481,6 +487,8 @@ archead_status archead_pack_create(const archead_desc *desc, void *stream, arche
   if ((e = dev_alloc(p, &p->s_v, (size_t)rc * 2)) != cudaSuccess) return fail(e);
   if ((e = dev_alloc(p, &p->s_b, G * rr * 2)) != cudaSuccess) return fail(e);
   if ((e = dev_alloc(p, &p->err, 16)) != cudaSuccess) return fail(e);
+  // (Enough for 128 tokens of any rank, so that no forward of those allocates them.)
+  if ((e = ensure_counters(p, prepass_pairs(kPrefillSplitPrepass, p->lr), s)) != cudaSuccess) return fail(e);
   if ((e = cudaMemsetAsync(p->err, 0, 16, s)) != cudaSuccess) return fail(e);
 
   // Canonical components: the V-indexed ones pass through temporaries on the
