@@ -40,8 +40,8 @@
 // of them MMAs) and, below 129 tokens, the conversion of the codes, which does
 // not depend on the tokens.  Qwen3-8B shape, before and now: 24 tokens 150 ->
 // 137 us, 64 tokens 246 -> 143, 4096 tokens 4.51 -> 3.66 ms; the paper's
-// format 200 tokens 318 -> 222 us, cross entropy of 2048 tokens 2.15 -> 1.74
-// ms; Gemma shape, cross entropy of 512 tokens 776 -> 667 us.
+// format 200 tokens 318 -> 221 us, cross entropy of 2048 tokens 2.15 -> 1.71
+// ms; Gemma shape, cross entropy of 512 tokens 776 -> 596 us.
 //
 // Epilogues: logits (each promotion thread stores one row of its tokens),
 // greedy partials (largest logit and its row per token over each warp's 32
@@ -898,7 +898,7 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
     // reduce over rows, with 4 rows x kCols/4 tokens per thread (16x256b): their
     // sums change shape through the tensor memory of the unit's last block.
     // (Promoting in that shape takes four factors a thread and half-height
-    // loads for every block: 4.27 against 3.35 ms for 4096 tokens, Qwen3-8B
+    // loads for every block: 4.27 against 3.56 ms for 4096 tokens, Qwen3-8B
     // shape.)  Cross entropy accumulates in base 2, its factors times log2 e.
     const int rt0 = lg * 32 + lane;
     const uint32_t lane_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + col0;
