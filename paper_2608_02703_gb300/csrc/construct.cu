@@ -383,11 +383,13 @@ __global__ void quantize_residual_sc4_kernel(const float *__restrict__ r, int64_
 // Group maxima come from the kLanes lanes holding a group (two halves, for g
 // = 256, meet in shared memory), the row maximum from the warps'; then one
 // thread per group takes its scale code, scale and reciprocal, while the next
-// row is on its way.  The one-warp-per-row kernel read r twice, 4 bytes a
+// row is on its way; four blocks a multiprocessor (151936 x 4096: 546 us;
+// three, as the registers would have it, 577; five 586; 3.4 TB/s without the
+// next row's loads).  The one-warp-per-row kernel read r twice, 4 bytes a
 // lane, and divided every value.
 constexpr int kSc4Threads = 256;
 template <int kNV>
-__global__ void __launch_bounds__(kSc4Threads) quantize_residual_sc4_rows_kernel(
+__global__ void __launch_bounds__(kSc4Threads, kNV <= 4 ? 4 : 2) quantize_residual_sc4_rows_kernel(
     const float4 *__restrict__ r, int64_t rows, int cols4, int lg, uint32_t *__restrict__ codes,
     uint8_t *__restrict__ qcodes, uint16_t *__restrict__ row_scale) {
   __shared__ float pmax[kSc4Threads * kNV / 8];  // per 32..128-wide piece of the row
