@@ -39,9 +39,9 @@
 // issuing warp's own instructions (two turns a stage: about 1400 cycles, 1070
 // of them MMAs) and, below 129 tokens, the conversion of the codes, which does
 // not depend on the tokens.  Qwen3-8B shape, before and now: 24 tokens 150 ->
-// 137 us, 64 tokens 246 -> 143, 4096 tokens 4.51 -> 3.66 ms; the paper's
+// 132 us, 64 tokens 246 -> 140, 4096 tokens 4.51 -> 3.66 ms; the paper's
 // format 200 tokens 318 -> 221 us, cross entropy of 2048 tokens 2.15 -> 1.71
-// ms; Gemma shape, cross entropy of 512 tokens 776 -> 596 us.
+// ms; Gemma shape, cross entropy of 512 tokens 776 -> 590 us.
 //
 // Epilogues: logits (each promotion thread stores one row of its tokens),
 // greedy partials (largest logit and its row per token over each warp's 32
@@ -83,14 +83,14 @@ struct PfGeom {
   static constexpr int kAParts = TM == 256 ? 2 : 1;  // an A stage is released in parts (256 tokens: halves)
   static constexpr int kBoxBytes = NT * 64 * 2;      // one TMA box of x: 64 of d
   static constexpr int kXBytes = 2 * kBoxBytes;
-  static constexpr int kXS = TM == 64 ? 8 : TM == 128 ? 5 : 5;
+  static constexpr int kXS = TM == 64 ? 8 : TM == 128 ? 4 : 5;
   static constexpr int kScaleOff = 2 * kChunkBytes;  // SC4: up to two byte rows of scale codes
   static constexpr int kCodeSlot = kScaleOff + 2 * kTileRows;
-  static constexpr int kCS = TM == 64 ? 11 : TM == 128 ? 7 : 7;
+  static constexpr int kCS = TM == 64 ? 11 : TM == 128 ? 11 : 7;
   static constexpr int kCodeOff = kXS * kXBytes;
   static constexpr int kBarOff = kCodeOff + kCS * kCodeSlot;
   static constexpr int kBars = 2 * kXS + 2 * kCS + kConv * (1 + kAParts) + 2 * kNB + 1;
-  static constexpr int kSmem = 1024 + kBarOff + kBars * 8 + 16;
+  static constexpr int kSmem = (TM == 128 ? 1024 : 0) + kBarOff + kBars * 8 + 16;
   // Registers a thread of the producer/MMA warpgroup, the converters and the
   // promotion warpgroups (launched with the largest multiple of 8 that fits);
   // their sum is that of the launch.
@@ -99,6 +99,12 @@ struct PfGeom {
   static constexpr int kRegsP = TM == 64 ? 128 : TM == 128 ? 112 : 160;
   static_assert(128 * (kRegs0 + kConv * kRegsC + kPromo * kRegsP) <= 65536 / kThreads / 8 * 8 * kThreads, "registers");
   static_assert(kABase + kConv * 64 <= kPfTmemCols, "TMEM columns");
+  // A converter warpgroup waits for stage n in a code slot whose last stage, n
+  // - kCS, was another's.  What it knows is that the MMAs of stage n - 2 kConv
+  // are done (its own A stage was free for n - kConv); with fewer slots than
+  // that the slot's barrier could still be a phase behind, which its parity
+  // does not show.
+  static_assert(kCS >= 2 * kConv, "code slots");
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
 
@@ -455,8 +461,19 @@ template <int TM, int kMode, bool kSC4>
 __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const __grid_constant__ PrefillParams p) {
   using G = PfGeom<TM>;
   constexpr int NT = G::NT, kNB = G::kNB, kXS = G::kXS, kCS = G::kCS, kConv = G::kConv, kCols = G::kCols;
+  // The kernel has no static shared memory, so the dynamic window starts on a
+  // 1 KB boundary, which the 128-byte-swizzled boxes rely on (checked).  The
+  // 128-token instance rounds the address up all the same: with a base the
+  // compiler knows its INT8 form takes 203 us for 100 tokens against 174 (the
+  // 64-token instance gains 3 %).
   extern __shared__ uint8_t pf_smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
+  uint8_t *smem = pf_smem_raw;
+  if constexpr (TM == 128)
+    smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(pf_smem_raw) + 1023) & ~(uintptr_t)1023);
+  if ((smem_u32(smem) & 1023u) != 0) {
+    if (threadIdx.x == 0) atomicOr(p.err, kErrLayout);
+    return;
+  }
   uint64_t *x_full = reinterpret_cast<uint64_t *>(smem + G::kBarOff);
   uint64_t *x_empty = x_full + kXS;
   uint64_t *c_full = x_empty + kXS;
