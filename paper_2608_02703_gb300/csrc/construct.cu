@@ -578,7 +578,9 @@ void launch_quantize_rows(const float *x, int64_t n, int qmax, int8_t *codes, ui
 cudaError_t launch_quantize_columns(const float *x, int64_t rows, int64_t cols, int64_t gr, int qmax, int8_t *codes,
                                     uint16_t *scales, cudaStream_t s) {
   const int64_t groups = rows / gr;
-  if (cols % 4 == 0 && cols <= 1024 && gr >= 4 * kColSlices && groups <= 65535 && aligned(x, 16) && aligned(codes, 4)) {
+  // (Below a million values one launch costs less than three.)
+  if (rows * cols >= 1 << 20 && cols % 4 == 0 && cols <= 1024 && gr >= 4 * kColSlices && groups <= 65535 &&
+      aligned(x, 16) && aligned(codes, 4)) {
     const int cols4 = (int)(cols / 4);
     const dim3 grid(kColSlices, (unsigned)groups);
     const float4 *x4 = reinterpret_cast<const float4 *>(x);
