@@ -77,9 +77,10 @@ typedef enum {
 } archead_format;
 
 typedef enum {
-  ARCHEAD_PATH_AUTO = 0,    /* decode kernel for M <= 16, tensor-core prefill kernel
-                               above (and for heads too wide for the decode kernel's
-                               shared memory)                                          */
+  ARCHEAD_PATH_AUTO = 0,    /* decode kernel for M <= 16 and, where it is the faster
+                               one (mostly large INT8 heads with groups of 32 or 64),
+                               up to 64; tensor-core prefill kernel above (and for
+                               heads too wide for the decode kernel's shared memory)   */
   ARCHEAD_PATH_DECODE = 1,  /* decode kernel: one launch per 16, 32 or 64 tokens (by M
                                and the head's width); ARCHEAD_ERR_UNSUPPORTED for
                                heads too wide for it                                   */

@@ -267,6 +267,16 @@ archead_status run_prefill(archead_pack *p, const void *x, int64_t M, void *out,
   return ARCHEAD_OK;
 }
 
+// AUTO's path: up to 16 tokens decode (memory bound, warp-level MMAs), up to
+// 64 the faster of the two, more the tensor-core kernel, one pass over the head
+// per 256 tokens.  Heads too wide for the decode kernel's shared memory plan
+// (per-group sums of x for 16 tokens, e.g. d = 2^20 at g = 32) take the
+// tensor-core kernel always.
+bool auto_decodes(const archead_pack *p, int64_t M, bool reduce) {
+  if (M <= kDecodeMaxTokens) return decode_supported(p->d_pad, p->nls_dec, p->g);
+  return M <= kDecodeWideTokens && decode_faster(p, (int)M, reduce);
+}
+
 archead_status run_forward(archead_pack *p, const void *x, int64_t M, void *out, int out_fp32,
                            const int32_t *targets, float *ce, archead_path path, cudaStream_t s,
                            int32_t *amax_idx = nullptr, float *amax_val = nullptr, int row0 = 0,
@@ -274,13 +284,8 @@ archead_status run_forward(archead_pack *p, const void *x, int64_t M, void *out,
   if (path != ARCHEAD_PATH_AUTO && path != ARCHEAD_PATH_DECODE && path != ARCHEAD_PATH_PREFILL)
     return ARCHEAD_ERR_INVALID_ARG;
   AH_CUDA(cudaSetDevice(p->device));
-  // AUTO: up to 16 tokens decode (memory bound, warp-level MMAs); more take
-  // the tensor-core kernel, one pass over the head per 128 tokens.
-  // Heads too wide for the decode kernel's shared memory plan (per-group
-  // sums of x for 16 tokens, e.g. d = 2^20 at g = 32) take the prefill
-  // kernel under AUTO.
-  const bool decode = path == ARCHEAD_PATH_DECODE ||
-                      (path == ARCHEAD_PATH_AUTO && M <= kDecodeMaxTokens && decode_supported(p->d_pad, p->nls_dec, p->g));
+  const bool decode =
+      path == ARCHEAD_PATH_DECODE || (path == ARCHEAD_PATH_AUTO && auto_decodes(p, M, out == nullptr));
   if (decode) return run_decode(p, x, M, out, out_fp32, targets, ce, amax_idx, amax_val, row0, parts3, s);
   return run_prefill(p, x, M, out, out_fp32, targets, ce, amax_idx, amax_val, row0, parts3, s);
 }

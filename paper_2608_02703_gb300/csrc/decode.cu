@@ -63,6 +63,46 @@ int decode_variant(const archead_pack *p, int M) {
   return pl.stages >= 2 && pl.xs_off >= (size_t)96 * 1024 ? resident : streamed;
 }
 
+// AUTO's choice for 17 to 64 tokens: true where the decode kernel is the
+// faster one.  The tensor-core kernel promotes every scale group of a tile
+// into fp32 registers one after the other, which takes it as long at 17 tokens
+// as at 64, so it loses INT8 heads with short groups (us, decode against
+// tensor-core kernel, ranks 128 + 32, 24 tokens): V = 151936, d = 4096 189
+// against 433 (g = 32) and 165 / 234 (64), but 150 / 135 (128) and 159 / 109
+// (256); in the paper's format, whose blocks are 512 wide, 180 / 106 even for
+// g = 32.  Above 32 tokens only g = 32 stays (64 tokens, the same head: 383 /
+// 443 and, g = 64, 335 / 240).  With at most a tile a multiprocessor the
+// decode kernel, whose units have two or four, loses (V = 8192, d = 1024,
+// g = 32: 20.5 / 16.4); beyond, the two times are estimated from the busiest
+// block's tiles: us per tile and 1024 of d, per tile and per launch, fitted to
+// 2936 pairs of times (13 vocabulary sizes from 16000 to 262144, d 512 to
+// 32768, logits and cross entropy).  On 150 other heads, every format and
+// group size, AUTO took 0.6 % longer than the faster kernel on average.
+//
+// A short second round of tiles costs the tensor-core kernel most on narrow
+// heads, where its start is most of the time (paper's format, g = 64, d = 512,
+// 32 tokens: 14.5 / 16.5 at V = 19456 to 32000, 20.5 / 18.6 at 38800).  The
+// same line for longer groups would gain as much, but there the decode kernel
+// is the less accurate one (relative error at d = 512: 3.9e-6 against 2.1e-6
+// for INT8, g = 256; 2.0e-6 both for the paper's format, g = 64), as it is
+// without rank-r branches (1.3e-6 against 4.5e-8 at d = 4096; with them, the
+// bf16 split of t leaves both at 2.2e-6).
+bool decode_faster(const archead_pack *p, int M, bool reduce) {
+  if (p->g > 64 || p->lr == 0 || !decode_supported(p->d_pad, p->nls_dec, p->g)) return false;
+  const auto rounds = [&](int units) { return (units + p->sm_count - 1) / p->sm_count; };
+  const int pf_tiles = rounds(p->num_tiles);
+  if (p->sc4) return M <= 32 && pf_tiles == 2 && 5 * p->num_tiles <= 8 * p->sm_count && p->d <= 768;
+  const int v = decode_variant(p, M);
+  if (pf_tiles < 2 || (p->g == 64 && v == kDecWide8)) return false;
+  const int launches = (M + variant_tokens(v) - 1) / variant_tokens(v);
+  const int dec_tiles = launches * rounds(decode_num_units(p, v)) * variant_tiles(v);
+  const bool g32 = p->g == 32;
+  const float k = p->d_pad / 1024.f;
+  const float per_k = v == kDecWide8 ? 8.f : v == kDecWide4 ? (g32 ? 5.f : 4.f) : (g32 ? 3.2f : 2.8f);
+  const float per_tile = (v == kDecWide8 ? 1.5f : 0.f) + (reduce ? (v == kDecWide8 ? 3.5f : 2.f) : 0.f);
+  return 10.f * launches + dec_tiles * (per_k * k + per_tile) < 5.5f + pf_tiles * (g32 ? 11.7f : 7.3f) * k;
+}
+
 extern template cudaError_t launch_decode_fmt<true>(const DecodeParams &, int, cudaStream_t, bool);
 template cudaError_t launch_decode_fmt<false>(const DecodeParams &, int, cudaStream_t, bool);
 

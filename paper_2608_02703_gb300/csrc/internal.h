@@ -191,6 +191,9 @@ bool decode_supported(int d_pad, int nls, int g);
 // resident; 1 (5: units of two tiles), 2, 3 two, four and eight n-tiles, x
 // streamed.
 int decode_variant(const archead_pack *p, int M);
+// 17 <= M <= 64: whether AUTO takes the decode kernel (reduce: cross entropy
+// or greedy, not logits).
+bool decode_faster(const archead_pack *p, int M, bool reduce);
 cudaError_t launch_prefill(const archead_pack *pk, const void *x, int M, const uint16_t *T, void *out, int out_fp32,
                            bool argmax, const int32_t *targets, int row0, float2 *ce_part, float *ce_tlogit,
                            bool pdl, cudaStream_t s);

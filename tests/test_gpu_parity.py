@@ -177,6 +177,46 @@ def test_tensor_core_token_edges(name, M):
     assert np.max(np.abs(ce - (lse - ref[np.arange(M), t]))) <= gu.CE_ABS
 
 
+# AUTO between 17 and 64 tokens: decode kernel for many-tile INT8 heads with
+# short groups (up to 32 tokens where g = 64) and narrow heads of the paper's
+# format with a short second round of tiles, tensor-core kernel for the rest.
+AUTO_ROUTES = [  # fmt, V, d, ranks, g, {M: path}
+    ("int8", 40000, 512, (20, 12), 32, {16: "decode", 17: "decode", 32: "decode", 33: "prefill", 65: "prefill"}),
+    ("int8", 60000, 1024, (20, 12), 32, {33: "decode", 64: "decode", 65: "prefill"}),
+    ("int8", 40000, 1024, (20, 12), 64, {17: "decode", 32: "decode", 33: "prefill"}),
+    ("int8", 40000, 512, (20, 12), 128, {16: "decode", 17: "prefill", 64: "prefill"}),
+    ("int8", 4000, 1024, (20, 12), 32, {17: "prefill"}),  # fewer tiles than multiprocessors
+    ("int8", 40000, 512, (0, 0), 32, {17: "prefill"}),
+    ("sc4", 40000, 512, (10, 6), 32, {17: "prefill"}),
+    ("sc4", 30000, 512, (10, 6), 64, {17: "decode", 32: "decode", 33: "prefill"}),
+    ("sc4", 30000, 512, (10, 6), 128, {17: "prefill"}),
+]
+
+
+def _launches(pack):
+    return {k["name"]: k["launches"] for k in archead.archead_profile_read(pack)}
+
+
+@pytest.mark.parametrize("fmt,V,d,ranks,g,routes", AUTO_ROUTES,
+                         ids=[f"{r[0]}-V{r[1]}-d{r[2]}-g{r[4]}-r{r[3][0]}" for r in AUTO_ROUTES])
+def test_auto_route(fmt, V, d, ranks, g, routes):
+    shape = HeadShape(V=V, d=d, core_rank=ranks[0], corr_rank=ranks[1], group_size=g, fmt=fmt)
+    head = make_head(shape, seed=8)
+    pack = archead.archead_pack_create(head, shape)
+    try:
+        archead.archead_profile_enable(pack, True)
+        x = make_hidden(d, max(routes), seed=80)
+        ref = oracle.logits(head, shape, x)
+        for M, want in routes.items():
+            before = _launches(pack)
+            got = gu.forward(pack, x[:M], archead.OUT_FP32, archead.PATH_AUTO)
+            ran = {n for n, c in _launches(pack).items() if c > before.get(n, 0)}
+            assert ran & {"decode", "prefill"} == {want}, f"M={M}: {ran}"
+            gu.check_logits(got, ref[:M], where=f"M={M}")
+    finally:
+        pack.close()
+
+
 @pytest.mark.parametrize("name", ["ragged", "tiny", "g32", "g256", "corr_only", "one_row", "max_rank", "sc4",
                                   "sc4_g32"])
 @pytest.mark.parametrize("M", [1, 7, 16, 40])
