@@ -138,6 +138,71 @@ ForwardPlan plan_decode(archead_pack *p, int64_t M, bool ce) {
   return f;
 }
 
+struct PrefillPlan {
+  size_t t_off = 0, ce_part_off = 0, tlogit_off = 0, partial_off = 0, total = 0;
+  bool split_pre = false;
+};
+
+// The same on the prefill path.  Few tokens take the pre-pass that splits d
+// over blocks (the tensor-core one runs M / 64 blocks per 32 columns, each
+// over the whole of d).
+PrefillPlan plan_prefill(archead_pack *p, int64_t M, bool ce) {
+  PrefillPlan f;
+  Carve c;
+  f.t_off = c.take((size_t)M * std::max(2 * p->lr, 64) * 2);
+  if (ce) {
+    f.ce_part_off = c.take((size_t)p->num_tiles * prefill_parts_per_vt() * M * sizeof(float2));
+    f.tlogit_off = c.take((size_t)M * sizeof(float));
+  }
+  f.split_pre = M <= kPrefillSplitPrepass;
+  if (f.split_pre) f.partial_off = c.take(prepass_partial_bytes((int)M, p->lr, p->d));
+  f.total = c.off;
+  return f;
+}
+
+// AUTO's path: up to 16 tokens decode (memory bound, warp-level MMAs), up to
+// 64 the faster of the two, more the tensor-core kernel, one pass over the head
+// per 256 tokens.  Heads too wide for the decode kernel's shared memory plan
+// (per-group sums of x for 16 tokens, e.g. d = 2^20 at g = 32) take the
+// tensor-core kernel always.
+bool auto_decodes(const archead_pack *p, int64_t M, bool reduce) {
+  if (M <= kDecodeMaxTokens) return decode_supported(p->d_pad, p->nls_dec, p->g);
+  return M <= kDecodeWideTokens && decode_faster(p, (int)M, reduce);
+}
+
+bool capturing(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+  cudaGetLastError();  // the legacy stream while another one is captured
+  return true;
+}
+
+// Workspace for a forward over M tokens that needs `bytes`, and, the first
+// time that a pack sees so many, for every forward with fewer, whatever its
+// output (logits or per-slice partials): a graph captured after a warm-up with
+// the most tokens never meets a growth.  Fewer tokens can need more, since the
+// decode kernel leaves up to twice the partials a tile and the split pre-pass
+// leaves sums (cross entropy, V = 262144, d = 4096, g = 64: 1.6 MB at 24
+// tokens, 2.2 at 16).  The most of each kernel instance, launch count and
+// pre-pass is at the listed counts.  A call under capture takes what fits.
+cudaError_t reserve_workspace(archead_pack *p, size_t bytes, int64_t M, cudaStream_t s) {
+  static_assert(kDecodeMaxTokens == 16 && kDecodeWideTokens == 64 && kPrefillSplitPrepass == 128, "counts below");
+  const int upto = (int)std::min<int64_t>(M, kPrefillSplitPrepass);
+  int reserved = p->reserved_tokens;
+  if (upto > reserved && !capturing(s)) {
+    for (int m : {8, 16, 32, 48, 64, 128}) {
+      for (bool reduce : {false, true})
+        bytes = std::max(bytes, auto_decodes(p, m, reduce) ? plan_decode(p, m, reduce).total
+                                                           : plan_prefill(p, m, reduce).total);
+      reserved = m;
+      if (m >= upto) break;
+    }
+  }
+  cudaError_t e = ensure_workspace(p, bytes, s);
+  if (e == cudaSuccess) p->reserved_tokens = reserved;
+  return e;
+}
+
 template <typename T>
 T *at(void *base, size_t off) {
   return reinterpret_cast<T *>(static_cast<char *>(base) + off);
@@ -160,7 +225,7 @@ archead_status run_decode(archead_pack *p, const void *x, int64_t M, void *out, 
   const bool ce_mode = out == nullptr;
   const bool greedy = amax_idx != nullptr;
   ForwardPlan f = plan_decode(p, M, ce_mode);
-  AH_CUDA(ensure_workspace(p, f.total, s));
+  AH_CUDA(reserve_workspace(p, f.total, M, s));
   AH_CUDA(ensure_counters(p, prepass_pairs((int)M, p->lr), s));
   PrepassParams pp = prepass_params(p, x, M);
   pp.partial = at<float>(p->ws, f.partial_off);
@@ -214,40 +279,21 @@ archead_status run_prefill(archead_pack *p, const void *x, int64_t M, void *out,
                            float *parts3, cudaStream_t s) {
   const bool ce_mode = out == nullptr;
   const bool greedy = amax_idx != nullptr;
-  Carve c;
-  const size_t t_off = c.take((size_t)M * std::max(2 * p->lr, 64) * 2);
-  size_t ce_part_off = 0, tlogit_off = 0;
-  if (ce_mode) {
-    ce_part_off = c.take((size_t)p->num_tiles * prefill_parts_per_vt() * M * sizeof(float2));
-    tlogit_off = c.take((size_t)M * sizeof(float));
-  }
-  // Few tokens: the pre-pass that splits d over blocks (the tensor-core one
-  // runs M / 64 blocks per 32 columns, each over the whole of d).
-  const bool split_pre = M <= kPrefillSplitPrepass;
-  size_t partial_off = 0, reserve = 0;
-  if (split_pre) {
-    partial_off = c.take(prepass_partial_bytes((int)M, p->lr, p->d));
-    AH_CUDA(ensure_counters(p, prepass_pairs((int)M, p->lr), s));
-  } else {
-    // A call with more tokens leaves room for any with fewer, partial sums
-    // included, so that those need no growth (under stream capture, say).
-    reserve = (size_t)kPrefillSplitPrepass * std::max(2 * p->lr, 64) * 2 + 256 +
-              prepass_partial_bytes(kPrefillSplitPrepass, p->lr, p->d);
-    if (ce_mode) reserve += (size_t)kPrefillSplitPrepass * (p->num_tiles * prefill_parts_per_vt() * sizeof(float2) + 4) + 512;
-  }
-  AH_CUDA(ensure_workspace(p, std::max(c.off, reserve), s));
+  const PrefillPlan f = plan_prefill(p, M, ce_mode);
+  AH_CUDA(reserve_workspace(p, f.total, M, s));
+  if (f.split_pre) AH_CUDA(ensure_counters(p, prepass_pairs((int)M, p->lr), s));
   PrepassParams pp = prepass_params(p, x, M);
   pp.ts = nullptr;
-  pp.T = at<uint16_t>(p->ws, t_off);
-  if (split_pre) {
-    pp.partial = at<float>(p->ws, partial_off);
+  pp.T = at<uint16_t>(p->ws, f.t_off);
+  if (f.split_pre) {
+    pp.partial = at<float>(p->ws, f.partial_off);
     pp.counters = p->counters;
     AH_CUDA(launch_prepass(pp, s, p));
   } else {
     AH_CUDA(launch_prepass_t(pp, p->lr_t, p->d_pad, s, p));
   }
-  float2 *ce_part = ce_mode ? at<float2>(p->ws, ce_part_off) : nullptr;
-  float *tlogit = ce_mode ? at<float>(p->ws, tlogit_off) : nullptr;
+  float2 *ce_part = ce_mode ? at<float2>(p->ws, f.ce_part_off) : nullptr;
+  float *tlogit = ce_mode ? at<float>(p->ws, f.tlogit_off) : nullptr;
   cudaEvent_t ev = nullptr;
   timer_begin(p, "prefill", s, &ev);
   // The kernel overlaps the pre-pass grid (programmatic dependent launch).
@@ -265,16 +311,6 @@ archead_status run_prefill(archead_pack *p, const void *x, int64_t M, void *out,
     if (e != cudaSuccess) return cuda_status(e);
   }
   return ARCHEAD_OK;
-}
-
-// AUTO's path: up to 16 tokens decode (memory bound, warp-level MMAs), up to
-// 64 the faster of the two, more the tensor-core kernel, one pass over the head
-// per 256 tokens.  Heads too wide for the decode kernel's shared memory plan
-// (per-group sums of x for 16 tokens, e.g. d = 2^20 at g = 32) take the
-// tensor-core kernel always.
-bool auto_decodes(const archead_pack *p, int64_t M, bool reduce) {
-  if (M <= kDecodeMaxTokens) return decode_supported(p->d_pad, p->nls_dec, p->g);
-  return M <= kDecodeWideTokens && decode_faster(p, (int)M, reduce);
 }
 
 archead_status run_forward(archead_pack *p, const void *x, int64_t M, void *out, int out_fp32,
