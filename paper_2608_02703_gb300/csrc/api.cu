@@ -92,8 +92,8 @@ cudaError_t ensure_workspace(archead_pack *p, size_t bytes, cudaStream_t s) {
 
 // Block counters of the pre-pass: zeroed once when (re)allocated; every
 // pre-pass call leaves them zero again.
+constexpr int kMinCounters = 1024;
 cudaError_t ensure_counters(archead_pack *p, int n, cudaStream_t s) {
-  (void)s;
   if (n <= p->counters_len) return cudaSuccess;
   cudaError_t e = cudaDeviceSynchronize();
   if (e != cudaSuccess) return e;
@@ -103,10 +103,12 @@ cudaError_t ensure_counters(archead_pack *p, int n, cudaStream_t s) {
     p->counters = nullptr;
     p->counters_len = 0;
   }
-  const int len = std::max(n, 1024);
+  const int len = std::max(n, kMinCounters);
   e = cudaMalloc(&p->counters, (size_t)len * 4);
   if (e != cudaSuccess) return e;
-  e = cudaMemset(p->counters, 0, (size_t)len * 4);
+  // (In the caller's stream: the legacy stream, which a plain memset takes,
+  // is not ordered before a non-blocking one.)
+  e = cudaMemsetAsync(p->counters, 0, (size_t)len * 4, s);
   if (e != cudaSuccess) return e;
   p->counters_len = len;
   p->owned_bytes += (int64_t)len * 4;
@@ -528,8 +530,13 @@ archead_status archead_pack_create(const archead_desc *desc, void *stream, arche
   if ((e = dev_alloc(p, &p->s_v, (size_t)rc * 2)) != cudaSuccess) return fail(e);
   if ((e = dev_alloc(p, &p->s_b, G * rr * 2)) != cudaSuccess) return fail(e);
   if ((e = dev_alloc(p, &p->err, 16)) != cudaSuccess) return fail(e);
-  // (Enough for 128 tokens of any rank, so that no forward of those allocates them.)
-  if ((e = ensure_counters(p, prepass_pairs(kPrefillSplitPrepass, p->lr), s)) != cudaSuccess) return fail(e);
+  // Counters for 128 tokens of any rank, so that no forward of those allocates
+  // them.  Cleared in the caller's stream and without waiting for the device,
+  // which another stream may be capturing a graph on.
+  const int counters = std::max(prepass_pairs(kPrefillSplitPrepass, p->lr), kMinCounters);
+  if ((e = dev_alloc(p, &p->counters, (size_t)counters * 4)) != cudaSuccess) return fail(e);
+  p->counters_len = counters;
+  if ((e = cudaMemsetAsync(p->counters, 0, (size_t)counters * 4, s)) != cudaSuccess) return fail(e);
   if ((e = cudaMemsetAsync(p->err, 0, 16, s)) != cudaSuccess) return fail(e);
 
   // Canonical components: the V-indexed ones pass through temporaries on the

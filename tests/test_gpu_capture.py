@@ -138,3 +138,26 @@ def test_capture_of_more_tokens_that_fit(new_pack):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(call.out, other.out)
+
+
+def test_pack_creation_while_another_stream_is_captured(new_pack):
+    """Pack creation waits for its own stream only, so it runs beside a capture."""
+    import torch
+
+    want = _Call(new_pack("wide"), "logits", 8)
+    want.run()
+    side = torch.cuda.Stream()
+    buf = torch.zeros(16, device="cuda")
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        buf += 1
+        pack = archead.archead_pack_create(_heads["wide"], SHAPES["wide"], stream=side)
+    try:
+        got = _Call(pack, "logits", 8)
+        got.run()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got.out, want.out) and bool((buf == 1).all())
+    finally:
+        pack.close()
