@@ -377,10 +377,10 @@ __global__ void quantize_residual_sc4_kernel(const float *__restrict__ r, int64_
   }
 }
 
-// The same for g = 32, 64, 128 or 256 and rows of up to 256 kNV float4
-// (cols <= 8192), 16-byte aligned: a block per row, the row held in
-// registers, so r is read once (5 bytes a value in all, which bounds it).
-// Group maxima come from the kLanes lanes holding a group (two halves, for g
+// The same for g = 32, 64, 128 or 256 and rows from several groups (see the
+// dispatch) up to 256 kNV float4 (cols <= 8192), 16-byte aligned: a block per
+// row, the row held in registers, so r is read once (5 bytes a value in all,
+// which bounds it).  Group maxima come from the kLanes lanes holding a group (two halves, for g
 // = 256, meet in shared memory), the row maximum from the warps'; then one
 // thread per group takes its scale code, scale and reciprocal, while the next
 // row is on its way; four blocks a multiprocessor (151936 x 4096: 546 us;
@@ -662,7 +662,12 @@ ARCHEAD_API archead_status archead_quantize_residual_sc4(const float *r, int64_t
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const int lg = group_size == 32 ? 5 : group_size == 64 ? 6 : group_size == 128 ? 7 : group_size == 256 ? 8 : 0;
   const int64_t per = cols / 4;  // float4 a row
-  if (lg && per <= 8 * kSc4Threads && aligned(r, 16) && aligned(codes, 4)) {
+  // A block per row costs 1.3 to 1.5 ns a row however short the row is, a warp
+  // per row 0.18 (g = 32), 0.28, 0.29, 0.43 (256) ns a group (151936 rows of
+  // 128 columns, g = 128: 199 us against 49; of 512: 217 / 170; of 768: 229 /
+  // 263; of 1024, g = 256: 240 / 260).
+  const int64_t block_cols = group_size == 32 ? 256 : group_size == 64 ? 384 : group_size == 128 ? 768 : 1024;
+  if (lg && cols >= block_cols && per <= 8 * kSc4Threads && aligned(r, 16) && aligned(codes, 4)) {
     if (per <= kSc4Threads) launch_sc4_rows<1>(r, rows, cols, lg, codes, scale_codes, row_scale, s);
     else if (per <= 2 * kSc4Threads) launch_sc4_rows<2>(r, rows, cols, lg, codes, scale_codes, row_scale, s);
     else if (per <= 4 * kSc4Threads) launch_sc4_rows<4>(r, rows, cols, lg, codes, scale_codes, row_scale, s);

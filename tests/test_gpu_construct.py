@@ -131,7 +131,10 @@ def test_quantiser_routes_agree_on_values_that_are_not_finite():
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
 
 
-@pytest.mark.parametrize("cols,g", [(32, 32), (1024, 256), (1056, 32), (2112, 64), (4096, 128), (8192, 256), (8256, 64)])
+@pytest.mark.parametrize("cols,g", [
+    (32, 32), (1024, 256), (1056, 32), (2112, 64), (4096, 128), (8192, 256), (8256, 64),
+    (224, 32), (256, 32), (320, 64), (384, 64), (640, 128), (768, 128), (768, 256),  # rows too short for a block, and enough
+])
 def test_sc4_residual_row_widths_bit_exact(cols, g):
     import torch
 
@@ -144,6 +147,37 @@ def test_sc4_residual_row_widths_bit_exact(cols, g):
     assert np.array_equal(rs.cpu().numpy().view(np.uint16), s)
     assert np.array_equal(rq.cpu().numpy(), q)
     assert np.array_equal(rc.cpu().numpy(), c)
+
+
+def _microseconds(call):
+    import torch
+
+    best = float("inf")
+    for _ in range(8):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            call()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 100)
+    return best
+
+
+@pytest.mark.parametrize("cols,g", [(128, 128), (256, 64), (768, 256), (512, 32), (1024, 128)])
+def test_sc4_residual_route_is_not_the_slower_one(cols, g):
+    """Against the general kernel (which unaligned buffers take); narrow rows
+    took a block each, up to 4.5 times as long."""
+    import torch
+
+    rows = 32000
+    x = torch.randn(rows * cols + 1, device="cuda")
+    rc = torch.empty(rows * cols, dtype=torch.int8, device="cuda")
+    rq = torch.empty((rows, cols // g), dtype=torch.uint8, device="cuda")
+    rs = torch.empty(rows, dtype=torch.int16, device="cuda")
+    t = [_microseconds(lambda: archead.archead_quantize_residual_sc4(
+        x[o:o + rows * cols].view(rows, cols), g, rc.view(rows, cols), rq, rs)) for o in (0, 1)]
+    assert t[0] <= 1.25 * t[1], f"{t[0]:.1f} us against {t[1]:.1f}"
 
 
 @pytest.mark.parametrize("rows,cols", [(1, 16), (3, 32), (8, 2), (129, 1040), (3, 34)])
