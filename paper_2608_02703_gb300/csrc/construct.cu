@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "device.cuh"
 #include "internal.h"
 
@@ -232,7 +234,7 @@ __global__ void __launch_bounds__(kColThreads) quantize_columns_kernel(const flo
 //      the group's codes, which are written only by pass 3;
 //   2: a block per group turns them into scales;
 //   3: codes.
-constexpr int kColSlices = 304;  // two row slices a multiprocessor
+constexpr int kColSlices = 304;  // most row slices of a group: two a multiprocessor
 __global__ void __launch_bounds__(256) column_maxima_kernel(const float4 *__restrict__ x, int cols4, int64_t gr,
                                                             int8_t *__restrict__ codes) {
   __shared__ float4 red[256];
@@ -582,11 +584,18 @@ cudaError_t launch_quantize_columns(const float *x, int64_t rows, int64_t cols, 
   if (rows * cols >= 1 << 20 && cols % 4 == 0 && cols <= 1024 && gr >= 4 * kColSlices && groups <= 65535 &&
       aligned(x, 16) && aligned(codes, 4)) {
     const int cols4 = (int)(cols / 4);
-    const dim3 grid(kColSlices, (unsigned)groups);
+    // Slices of at least the eight rows that a thread has in flight, as long as
+    // all groups' together are two a multiprocessor.  (304 for every group,
+    // nearly empty where groups are many: 200 groups of 1216 x 128 281 us
+    // against 64, of 2048 x 32 199 / 28.)
+    const int64_t full = gr / (8 * (256 / cols4));
+    const int64_t least = (kColSlices + groups - 1) / groups;
+    const int slices = (int)std::max(least, std::min<int64_t>(kColSlices, full));
+    const dim3 grid((unsigned)slices, (unsigned)groups);
     const float4 *x4 = reinterpret_cast<const float4 *>(x);
     column_maxima_kernel<<<grid, 256, 0, s>>>(x4, cols4, gr, codes);
     column_scales_kernel<<<dim3((unsigned)((cols + 31) / 32), (unsigned)groups), 256, 0, s>>>(
-        codes, (int)cols, gr, kColSlices, (float)qmax, scales);
+        codes, (int)cols, gr, slices, (float)qmax, scales);
     column_codes_kernel<<<grid, 256, 0, s>>>(x4, cols4, gr, (float)qmax, scales, reinterpret_cast<uint32_t *>(codes));
     return cudaGetLastError();
   }

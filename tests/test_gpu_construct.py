@@ -110,6 +110,7 @@ def _quantise_at(x, gr, gc, bits, offset):
     ((3, 32), (1, 32), 4), ((37, 192), (1, 64), 4), ((5, 1664), (1, 128), 8), ((9, 768), (1, 256), 5),  # rows
     ((511, 3), (511, 1), 8), ((512, 7), (512, 1), 8), ((4095, 16), (4095, 1), 5), ((4096, 16), (4096, 1), 8),
     ((20011, 13), (20011, 1), 8), ((1200, 24), (600, 1), 4),
+    ((5 * 1216, 180), (1216, 1), 8), ((40 * 2048, 16), (2048, 1), 8),  # several groups
     ((1215, 4), (1215, 1), 8), ((1216, 4), (1216, 1), 8), ((2432, 1024), (1216, 1), 5), ((9001, 200), (9001, 1), 8),  # columns
 ], ids=str)
 def test_quantiser_routes_bit_exact(shape, groups, bits, offset):
@@ -177,6 +178,20 @@ def test_sc4_residual_route_is_not_the_slower_one(cols, g):
     rs = torch.empty(rows, dtype=torch.int16, device="cuda")
     t = [_microseconds(lambda: archead.archead_quantize_residual_sc4(
         x[o:o + rows * cols].view(rows, cols), g, rc.view(rows, cols), rq, rs)) for o in (0, 1)]
+    assert t[0] <= 1.25 * t[1], f"{t[0]:.1f} us against {t[1]:.1f}"
+
+
+def test_column_route_of_many_groups_is_not_the_slower_one():
+    """Against the strips of eight columns (which unaligned buffers take)."""
+    import torch
+
+    gr, groups, cols = 2048, 200, 32
+    n = gr * groups * cols
+    x = torch.randn(n + 1, device="cuda")
+    codes = torch.empty((gr * groups, cols), dtype=torch.int8, device="cuda")
+    scales = torch.empty((groups, cols), dtype=torch.int16, device="cuda")
+    t = [_microseconds(lambda: archead.archead_quantize_symmetric(x[o:o + n].view(-1, cols), gr, 1, 8, codes, scales))
+         for o in (0, 1)]
     assert t[0] <= 1.25 * t[1], f"{t[0]:.1f} us against {t[1]:.1f}"
 
 
