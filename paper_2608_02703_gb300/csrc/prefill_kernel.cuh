@@ -389,9 +389,12 @@ __device__ __forceinline__ void quad_ce(const PrefillParams &p, float (&acc)[NT]
   const int ru = lane >> 2, cq = lane & 3;
   m0 += 64 * HH;
   // Target logits first: a token whose target is one of this warp's 32 rows
-  // takes its value from the thread holding it (rare, so the slow path is a
-  // warp-uniform branch).  Lane (ru, cq) reads the targets of the columns it
-  // ends with.
+  // takes its value from the thread holding it (a warp-uniform branch, taken
+  // for 64 * 32 / V of the warps' halves).  Lane (ru, cq) reads the targets of
+  // the columns it ends with; each thread then looks at its own 16 columns.
+  // (Two shuffles for each of the 64 columns, in some warp of most units at
+  // V = 32000, took up to half of the time: paper's format, d = 1024, 4096
+  // tokens 447 us, now 256.)
   int tg[2];
   bool hit = false;
 #pragma unroll
@@ -403,15 +406,12 @@ __device__ __forceinline__ void quad_ce(const PrefillParams &p, float (&acc)[NT]
   }
   if (__any_sync(0xffffffffu, hit)) {
 #pragma unroll
-    for (int col = 0; col < 64; ++col) {
-      const int owner = 4 * (col >> 3) + ((col >> 1) & 3);  // lane that read this column's target
-      const int r = __shfl_sync(0xffffffffu, tg[col & 1], owner);
-      if (r >= 0) {  // warp-uniform
-        const int i0 = 4 * (8 * HH + (col >> 3)) + (col & 1);
-        const float mine =
-            r & 16 ? (r & 8 ? acc[i0 + NT / 2 + 2] : acc[i0 + NT / 2]) : (r & 8 ? acc[i0 + 2] : acc[i0]);
-        const float v = __shfl_sync(0xffffffffu, mine, 4 * (r & 7) + ((col >> 1) & 3));
-        if (lane == owner) p.ce_tlogit[m0 + col] = v * kLn2;
+    for (int k = 0; k < 16; ++k) {  // the thread's columns, their targets from lane (k / 2, cq)
+      const int r = __shfl_sync(0xffffffffu, tg[k & 1], 4 * (k >> 1) + cq);
+      if (r >= 0 && (r & 7) == ru) {
+        const int i0 = quad_i0<NT, HH>(k);
+        const float v = r & 16 ? (r & 8 ? acc[i0 + NT / 2 + 2] : acc[i0 + NT / 2]) : (r & 8 ? acc[i0 + 2] : acc[i0]);
+        p.ce_tlogit[m0 + 8 * (k >> 1) + 2 * cq + (k & 1)] = v * kLn2;
       }
     }
   }

@@ -27,6 +27,21 @@ def to_dev(a: np.ndarray):
     return t.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
+def microseconds(call) -> float:
+    """Best of eight runs of ten calls each."""
+    t = torch()
+    best = float("inf")
+    for _ in range(8):
+        a, b = t.cuda.Event(enable_timing=True), t.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(10):
+            call()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) * 100)
+    return best
+
+
 def forward(pack, x_bits: np.ndarray, out_dtype=archead.OUT_FP32, path=archead.PATH_AUTO) -> np.ndarray:
     t = torch()
     M = x_bits.shape[0]

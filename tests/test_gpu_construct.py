@@ -150,21 +150,6 @@ def test_sc4_residual_row_widths_bit_exact(cols, g):
     assert np.array_equal(rc.cpu().numpy(), c)
 
 
-def _microseconds(call):
-    import torch
-
-    best = float("inf")
-    for _ in range(8):
-        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        a.record()
-        for _ in range(10):
-            call()
-        b.record()
-        b.synchronize()
-        best = min(best, a.elapsed_time(b) * 100)
-    return best
-
-
 @pytest.mark.parametrize("cols,g", [(128, 128), (256, 64), (768, 256), (512, 32), (1024, 128)])
 def test_sc4_residual_route_is_not_the_slower_one(cols, g):
     """Against the general kernel (which unaligned buffers take); narrow rows
@@ -176,7 +161,7 @@ def test_sc4_residual_route_is_not_the_slower_one(cols, g):
     rc = torch.empty(rows * cols, dtype=torch.int8, device="cuda")
     rq = torch.empty((rows, cols // g), dtype=torch.uint8, device="cuda")
     rs = torch.empty(rows, dtype=torch.int16, device="cuda")
-    t = [_microseconds(lambda: archead.archead_quantize_residual_sc4(
+    t = [gu.microseconds(lambda: archead.archead_quantize_residual_sc4(
         x[o:o + rows * cols].view(rows, cols), g, rc.view(rows, cols), rq, rs)) for o in (0, 1)]
     assert t[0] <= 1.25 * t[1], f"{t[0]:.1f} us against {t[1]:.1f}"
 
@@ -190,7 +175,7 @@ def test_column_route_of_many_groups_is_not_the_slower_one():
     x = torch.randn(n + 1, device="cuda")
     codes = torch.empty((gr * groups, cols), dtype=torch.int8, device="cuda")
     scales = torch.empty((groups, cols), dtype=torch.int16, device="cuda")
-    t = [_microseconds(lambda: archead.archead_quantize_symmetric(x[o:o + n].view(-1, cols), gr, 1, 8, codes, scales))
+    t = [gu.microseconds(lambda: archead.archead_quantize_symmetric(x[o:o + n].view(-1, cols), gr, 1, 8, codes, scales))
          for o in (0, 1)]
     assert t[0] <= 1.25 * t[1], f"{t[0]:.1f} us against {t[1]:.1f}"
 

@@ -217,6 +217,28 @@ def test_auto_route(fmt, V, d, ranks, g, routes):
         pack.close()
 
 
+@pytest.mark.parametrize("fmt,g", [("sc4", 64), ("int8", 64)])
+def test_targets_cost_the_cross_entropy_little(fmt, g):
+    """Per-shard cross-entropy partials with every target in the shard against
+    none: on a narrow head, picking the targets' logits out of the registers
+    once took as long as the rest."""
+    import torch
+
+    shape = HeadShape(V=20000, d=512, core_rank=10, corr_rank=6, group_size=g, fmt=fmt)
+    pack = archead.archead_pack_create(make_head(shape, seed=3), shape)
+    try:
+        M = 2048
+        x = gu.to_dev(make_hidden(shape.d, M, seed=4))
+        t = torch.randint(0, shape.V, (M,), dtype=torch.int32, device="cuda")
+        out = torch.empty((M, 3), dtype=torch.float32, device="cuda")
+        inside, outside = (gu.microseconds(lambda: archead.archead_forward_lse_partial(pack, x, M, tt, 0, out))
+                           for tt in (t, t + shape.V))
+        assert archead.archead_sync_status(pack) == archead.OK
+        assert inside <= 1.3 * outside, f"{inside:.1f} us against {outside:.1f}"
+    finally:
+        pack.close()
+
+
 @pytest.mark.parametrize("name", ["ragged", "tiny", "g32", "g256", "corr_only", "one_row", "max_rank", "sc4",
                                   "sc4_g32"])
 @pytest.mark.parametrize("M", [1, 7, 16, 40])
