@@ -395,23 +395,29 @@ __device__ __forceinline__ void quad_ce(const PrefillParams &p, float (&acc)[NT]
   // (Two shuffles for each of the 64 columns, in some warp of most units at
   // V = 32000, took up to half of the time: paper's format, d = 1024, 4096
   // tokens 447 us, now 256.)
-  int tg[2];
-  bool hit = false;
+  uint32_t tg = 0;  // row + 1 within the warp's 32 of column j's target in byte j, 0: elsewhere
 #pragma unroll
   for (int j = 0; j < 2; ++j) {
     const int m = m0 + 8 * ru + 2 * cq + j;
     const int64_t t64 = m < mend ? (int64_t)p.targets[m] - p.row0 - rbase : -1;  // row within the warp's 32
-    tg[j] = t64 >= 0 && t64 < 32 ? (int)t64 : -1;
-    hit |= tg[j] >= 0;
+    if (t64 >= 0 && t64 < 32) tg |= (uint32_t)(t64 + 1) << (8 * j);
   }
-  if (__any_sync(0xffffffffu, hit)) {
+  if (__any_sync(0xffffffffu, tg != 0)) {
+    // (With the whole address formed per column the INT8 128-token instance
+    // spilled 64 bytes and took up to 22 % longer.)
+    float *tl = p.ce_tlogit + m0 + 2 * cq;
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {  // the thread's columns, their targets from lane (k / 2, cq)
-      const int r = __shfl_sync(0xffffffffu, tg[k & 1], 4 * (k >> 1) + cq);
-      if (r >= 0 && (r & 7) == ru) {
-        const int i0 = quad_i0<NT, HH>(k);
-        const float v = r & 16 ? (r & 8 ? acc[i0 + NT / 2 + 2] : acc[i0 + NT / 2]) : (r & 8 ? acc[i0 + 2] : acc[i0]);
-        p.ce_tlogit[m0 + 8 * (k >> 1) + 2 * cq + (k & 1)] = v * kLn2;
+    for (int k = 0; k < 16; k += 2) {  // the thread's columns, their targets from lane (k / 2, cq)
+      const uint32_t rs = __shfl_sync(0xffffffffu, tg, 4 * (k >> 1) + cq);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int r = (int)(rs >> (8 * j) & 255) - 1;
+        if (r >= 0 && (r & 7) == ru) {
+          const int i0 = quad_i0<NT, HH>(k + j);
+          const float v =
+              r & 16 ? (r & 8 ? acc[i0 + NT / 2 + 2] : acc[i0 + NT / 2]) : (r & 8 ? acc[i0 + 2] : acc[i0]);
+          tl[8 * (k >> 1) + j] = v * kLn2;
+        }
       }
     }
   }
