@@ -111,6 +111,10 @@ def _quantise_at(x, gr, gc, bits, offset):
     ((511, 3), (511, 1), 8), ((512, 7), (512, 1), 8), ((4095, 16), (4095, 1), 5), ((4096, 16), (4096, 1), 8),
     ((20011, 13), (20011, 1), 8), ((1200, 24), (600, 1), 4),
     ((5 * 1216, 180), (1216, 1), 8), ((40 * 2048, 16), (2048, 1), 8),  # several groups
+    # Kernels' outer loops several times over: rows, columns in three passes
+    # (one group, two), columns in strips.
+    ((20011, 1056), (1, 32), 4), ((262144, 4), (262144, 1), 8), ((40013, 128), (40013, 1), 8),
+    ((2 * 6000, 1024), (6000, 1), 8), ((40000, 16), (40000, 1), 8),
     ((1215, 4), (1215, 1), 8), ((1216, 4), (1216, 1), 8), ((2432, 1024), (1216, 1), 5), ((9001, 200), (9001, 1), 8),  # columns
 ], ids=str)
 def test_quantiser_routes_bit_exact(shape, groups, bits, offset):
@@ -130,6 +134,56 @@ def test_quantiser_routes_agree_on_values_that_are_not_finite():
     x[4, 9] = 3e38
     a, b = _quantise_at(x, 1, 64, 4, 0), _quantise_at(x, 1, 64, 4, 1)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+def _residual_at(x, g, offset):
+    """The paper's residual quantiser on buffers that start `offset` elements past an allocation."""
+    import torch
+
+    R, C = x.shape
+    xd = torch.empty(R * C + offset, dtype=torch.float32, device="cuda")
+    xd[offset:] = _dev(x).view(-1)
+    rc = torch.zeros(R * C + offset, dtype=torch.int8, device="cuda")
+    rq = torch.zeros((R, C // g), dtype=torch.uint8, device="cuda")
+    rs = torch.zeros(R, dtype=torch.int16, device="cuda")
+    view = rc[offset:].view(R, C)
+    archead.archead_quantize_residual_sc4(xd[offset:].view(R, C), g, view, rq, rs)
+    return view.cpu().numpy(), rq.cpu().numpy(), rs.cpu().numpy().view(np.uint16)
+
+
+def _not_finite(seed, shape):
+    x = _edge_values(seed, shape)
+    x[1, ::7] = np.nan
+    x[2, 3] = np.inf
+    x[3] = np.nan
+    x[4, 9] = 3e38
+    x[5, 2:5] = -np.inf
+    x[:, 6] = np.nan
+    return x
+
+
+@pytest.mark.parametrize("shape", [(1300, 12), (70000, 16), (9001, 120)])  # strips, three passes
+def test_column_routes_agree_on_values_that_are_not_finite(shape):
+    """Against the general kernel on the transpose (one group a row)."""
+    x = _not_finite(2, shape)
+    codes, scales = _quantise_at(x, shape[0], 1, 8, 0)
+    rc, rs = _quantise_at(np.ascontiguousarray(x.T), 1, shape[0], 8, 0)
+    assert np.array_equal(codes, rc.T) and np.array_equal(scales.ravel(), rs.ravel())
+
+
+@pytest.mark.parametrize("cols,g", [(512, 32), (1024, 256), (4096, 64)])
+def test_residual_routes_agree_on_values_that_are_not_finite(cols, g):
+    x = _not_finite(3, (9, cols))
+    for a, b in zip(_residual_at(x, g, 0), _residual_at(x, g, 1)):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("rows,cols,g", [(10007, 256, 32), (9731, 1056, 32), (9800, 1024, 256)])
+def test_sc4_residual_blocks_of_several_rows_bit_exact(rows, cols, g):
+    """More rows than blocks: the next row's loads and the shared memory of a row after another."""
+    x = _edge_values(rows, (rows, cols))
+    for a, b in zip(_residual_at(x, g, 0), oc.quantize_residual_sc4(x, g)):
+        assert np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("cols,g", [

@@ -177,6 +177,34 @@ def test_tensor_core_token_edges(name, M):
     assert np.max(np.abs(ce - (lse - ref[np.arange(M), t]))) <= gu.CE_ABS
 
 
+# Tokens whose last unit has a half without any (256-token units in halves of
+# a multiple of 16: 769 in halves of 112, 1121 of 128, 1793 of 128).
+@pytest.mark.parametrize("name,M", [
+    ("g32", 769), ("g128", 784), ("sc4_g32", 1121), ("core_only", 1152), ("sc4_ragged", 1793), ("group_int4", 1920),
+    ("many_tiles", 769), ("sc4_many_tiles", 769),
+])
+def test_units_with_an_empty_half(name, M):
+    shape = MANY_TILES.get(name) or SHAPES[name]
+    halves = 2 * ((M + 255) // 256)
+    nt = ((M + halves - 1) // halves + 15) // 16 * 16
+    assert (halves - 1) * nt >= M
+    if name in MANY_TILES and name not in _packs:
+        head = make_head(shape, seed=5)
+        _packs[name] = (archead.archead_pack_create(head, shape), head)
+    pack, head = get(name)
+    x = make_hidden(shape.d, M, seed=900 + M)
+    ref = oracle.logits(head, shape, x)
+    gu.check_logits(gu.forward(pack, x), ref, where=f"{name} M={M}")
+    idx, val = gu.forward_argmax(pack, x)
+    gu.check_greedy(idx, val, ref, where=f"{name} M={M}")
+    t = make_targets(shape.V, M, seed=M)
+    ce, st = gu.forward_ce(pack, x, t)
+    assert st == archead.OK
+    mx = ref.max(axis=1)
+    lse = mx + np.log(np.exp(ref - mx[:, None]).sum(axis=1))
+    assert np.max(np.abs(ce - (lse - ref[np.arange(M), t]))) <= gu.CE_ABS
+
+
 # AUTO between 17 and 64 tokens: decode kernel for many-tile INT8 heads with
 # short groups (up to 32 tokens where g = 64) and narrow heads of the paper's
 # format with a short second round of tiles, tensor-core kernel for the rest.
