@@ -28,7 +28,9 @@
  *    concurrent calls); successive calls may use different streams.  When a
  *    call needs a larger workspace than the pack holds, it synchronises the
  *    device before freeing the old one, so earlier calls on any stream are
- *    done with it.  Different packs are independent.
+ *    done with it.  A call that is not being captured leaves room for every
+ *    AUTO call of its kind (logits; or cross entropy, greedy and partials)
+ *    with fewer tokens.  Different packs are independent.
  *  - Faults detected on the device (an out-of-range target, a pipeline wait
  *    that gave up) are latched in a per-pack device error word and reported
  *    by archead_sync_status().

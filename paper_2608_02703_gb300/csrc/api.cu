@@ -152,13 +152,17 @@ PrefillPlan plan_prefill(archead_pack *p, int64_t M, bool ce) {
   PrefillPlan f;
   Carve c;
   f.t_off = c.take((size_t)M * std::max(2 * p->lr, 64) * 2);
+  // The split pre-pass's sums share their place with the partials of the
+  // output, which no block writes before it has waited for the pre-pass grid's
+  // end (t is part of every logit).
+  Carve sums = c;
+  f.split_pre = M <= kPrefillSplitPrepass;
+  if (f.split_pre) f.partial_off = sums.take(prepass_partial_bytes((int)M, p->lr, p->d));
   if (ce) {
     f.ce_part_off = c.take((size_t)p->num_tiles * prefill_parts_per_vt() * M * sizeof(float2));
     f.tlogit_off = c.take((size_t)M * sizeof(float));
   }
-  f.split_pre = M <= kPrefillSplitPrepass;
-  if (f.split_pre) f.partial_off = c.take(prepass_partial_bytes((int)M, p->lr, p->d));
-  f.total = c.off;
+  f.total = std::max(c.off, sums.off);
   return f;
 }
 
@@ -180,28 +184,28 @@ bool capturing(cudaStream_t s) {
 }
 
 // Workspace for a forward over M tokens that needs `bytes`, and, the first
-// time that a pack sees so many, for every forward with fewer, whatever its
-// output (logits or per-slice partials): a graph captured after a warm-up with
-// the most tokens never meets a growth.  Fewer tokens can need more, since the
-// decode kernel leaves up to twice the partials a tile and the split pre-pass
-// leaves sums (cross entropy, V = 262144, d = 4096, g = 64: 1.6 MB at 24
-// tokens, 2.2 at 16).  The most of each kernel instance, launch count and
-// pre-pass is at the listed counts.  A call under capture takes what fits.
-cudaError_t reserve_workspace(archead_pack *p, size_t bytes, int64_t M, cudaStream_t s) {
+// time that a pack sees so many, for every forward of that kind (logits; or
+// cross entropy, greedy and logits) with fewer: a graph captured after a
+// warm-up with the most tokens then meets no growth.  Fewer tokens can need
+// more, since the decode kernel leaves up to twice the partials a tile and the
+// split pre-pass leaves sums (cross entropy, V = 262144, d = 4096, g = 64:
+// 1.6 MB at 24 tokens, 2.2 at 16).  The most of each kernel instance, launch
+// count and pre-pass is at the listed counts.  A call under capture takes what
+// fits.
+cudaError_t reserve_workspace(archead_pack *p, size_t bytes, int64_t M, bool reduce, cudaStream_t s) {
   static_assert(kDecodeMaxTokens == 16 && kDecodeWideTokens == 64 && kPrefillSplitPrepass == 128, "counts below");
   const int upto = (int)std::min<int64_t>(M, kPrefillSplitPrepass);
-  int reserved = p->reserved_tokens;
-  if (upto > reserved && !capturing(s)) {
-    for (int m : {8, 16, 32, 48, 64, 128}) {
-      for (bool reduce : {false, true})
-        bytes = std::max(bytes, auto_decodes(p, m, reduce) ? plan_decode(p, m, reduce).total
-                                                           : plan_prefill(p, m, reduce).total);
-      reserved = m;
-      if (m >= upto) break;
+  const bool more = upto > p->reserved_tokens[reduce] && !capturing(s);
+  if (more) {
+    for (int end : {8, 16, 32, 48, 64, 128}) {
+      const int m = std::min(end, upto);
+      for (int kind = 0; kind <= (int)reduce; ++kind)
+        bytes = std::max(bytes, auto_decodes(p, m, kind) ? plan_decode(p, m, kind).total : plan_prefill(p, m, kind).total);
+      if (m == upto) break;
     }
   }
   cudaError_t e = ensure_workspace(p, bytes, s);
-  if (e == cudaSuccess) p->reserved_tokens = reserved;
+  if (e == cudaSuccess && more) p->reserved_tokens[reduce] = upto;
   return e;
 }
 
@@ -227,7 +231,7 @@ archead_status run_decode(archead_pack *p, const void *x, int64_t M, void *out, 
   const bool ce_mode = out == nullptr;
   const bool greedy = amax_idx != nullptr;
   ForwardPlan f = plan_decode(p, M, ce_mode);
-  AH_CUDA(reserve_workspace(p, f.total, M, s));
+  AH_CUDA(reserve_workspace(p, f.total, M, ce_mode, s));
   AH_CUDA(ensure_counters(p, prepass_pairs((int)M, p->lr), s));
   PrepassParams pp = prepass_params(p, x, M);
   pp.partial = at<float>(p->ws, f.partial_off);
@@ -282,7 +286,7 @@ archead_status run_prefill(archead_pack *p, const void *x, int64_t M, void *out,
   const bool ce_mode = out == nullptr;
   const bool greedy = amax_idx != nullptr;
   const PrefillPlan f = plan_prefill(p, M, ce_mode);
-  AH_CUDA(reserve_workspace(p, f.total, M, s));
+  AH_CUDA(reserve_workspace(p, f.total, M, ce_mode, s));
   if (f.split_pre) AH_CUDA(ensure_counters(p, prepass_pairs((int)M, p->lr), s));
   PrepassParams pp = prepass_params(p, x, M);
   pp.ts = nullptr;

@@ -140,7 +140,7 @@ struct archead_pack {
   // workspace (grown on demand) and the pre-pass block counters (kept zero)
   void *ws = nullptr;
   size_t ws_bytes = 0;
-  int reserved_tokens = 0;  // every forward of up to so many tokens fits
+  int reserved_tokens[2] = {0, 0};  // logits, other outputs: every forward of up to so many tokens fits
   int *counters = nullptr;
   int counters_len = 0;
   // host staging for archead_forward_host
