@@ -111,9 +111,8 @@ __global__ void __launch_bounds__(256) quantize_rows_kernel(const float4 *__rest
   }
 }
 
-// Groups of gr rows of one column (the core factors: gr = all rows; the
-// correction's right factor: gr = g), for any number of columns and any
-// alignment.  A cluster of blocks takes one group of rows of eight adjacent
+// Groups of gr >= 512 rows of one column (the core factors: gr = all rows),
+// for any number of columns and any alignment.  A cluster of blocks takes one group of rows of eight adjacent
 // columns (one 32-byte sector of a row), each block a slice of the rows:
 // column maxima over its slice, the maximum over the cluster through
 // distributed shared memory, then the codes, x coming mostly from L2 the
@@ -311,7 +310,7 @@ __global__ void __launch_bounds__(256) column_codes_kernel(const float4 *__restr
 }
 
 // One warp per scale group of gr x gc elements of x [rows][cols]: the shapes
-// that the two kernels above do not take.
+// that the kernels above do not take.
 __global__ void quantize_symmetric_kernel(const float *__restrict__ x, int64_t rows, int64_t cols, int64_t gr,
                                           int64_t gc, int qmax, int8_t *__restrict__ codes,
                                           uint16_t *__restrict__ scales) {
@@ -568,7 +567,8 @@ archead_status fail_cuda(cudaError_t e) {
 bool aligned(const void *p, size_t n) { return (reinterpret_cast<uintptr_t>(p) & (n - 1)) == 0; }
 
 // Blocks for grid-stride kernels: enough for several a multiprocessor, so
-// that a thread's independent loads are in flight on every one of them.
+// that a thread's independent loads are in flight on every one of them.  (As
+// kColSlices, sized for 152; the results do not depend on it.)
 unsigned stream_grid(int64_t blocks) { return (unsigned)(blocks < 1 ? 1 : blocks < 152 * 32 ? blocks : 152 * 32); }
 
 template <int kGc>

@@ -12,11 +12,11 @@
 //     into exact bf16 integers and stores them as the A operand in tensor
 //     memory: the code layout is that of m16n8k16 fragments, which is the
 //     register layout of tcgen05.st.16x128b;
-//   - one thread issues eight tcgen05.mma (kind::f16, 128 x 64 or 128 x 16, A
-//     from TMEM, B = x from shared memory, fp32 accumulate) into a ring of
-//     TMEM accumulators; with 256 tokens, eight for each half of them, so that
-//     each conversion serves 256 tokens and one half's finished group is
-//     drained while the other computes;
+//   - one thread issues eight tcgen05.mma (kind::f16, 128 rows x nt tokens x
+//     16, nt a multiple of 16 up to 128, A from TMEM, B = x from shared memory,
+//     fp32 accumulate) into a ring of TMEM accumulators; with 256 tokens, eight
+//     for each half of them, so that each conversion serves 256 tokens and one
+//     half's finished group is drained while the other computes;
 //   - promotion warps read each finished block with tcgen05.ld and add
 //     s[row, group] * partial to fp32 registers (group-wise scales cannot be
 //     folded into exact bf16 operands).
@@ -37,11 +37,14 @@
 // measured tensor peak.  With A in TMEM an MMA of N tokens takes about N / 2 +
 // 5 cycles (measured alone: 39 for 64, 67 for 128), and what is left is the
 // issuing warp's own instructions (two turns a stage: about 1400 cycles, 1070
-// of them MMAs) and, below 129 tokens, the conversion of the codes, which does
-// not depend on the tokens.  Qwen3-8B shape, before and now: 24 tokens 150 ->
-// 132 us, 64 tokens 246 -> 140, 4096 tokens 4.51 -> 3.66 ms; the paper's
-// format 200 tokens 318 -> 221 us, cross entropy of 2048 tokens 2.15 -> 1.71
-// ms; Gemma shape, cross entropy of 512 tokens 776 -> 590 us.
+// of them MMAs).  Up to 64 tokens no role is busy all the time: an issuer's
+// turn takes some 740 cycles for 200 to 310 of MMAs, and what does not depend
+// on the tokens (the conversion of the codes, the promotion of the instance's
+// whole width, group by group, the boundaries of units) shares the rest.
+// Qwen3-8B shape, before and now: 24 tokens 150 -> 132 us, 64 tokens 246 ->
+// 140, 4096 tokens 4.51 -> 3.66 ms; the paper's format 200 tokens 318 -> 223
+// us, cross entropy of 2048 tokens 2.15 -> 1.65 ms; Gemma shape, cross entropy
+// of 512 tokens 776 -> 570 us.
 //
 // Epilogues: logits (each promotion thread stores one row of its tokens),
 // greedy partials (largest logit and its row per token over each warp's 32
@@ -67,9 +70,10 @@ constexpr float kLn2 = 0.6931471805599453f;    // ln(2)
 // Instance geometry for TM tokens a unit, in kH halves of NT.  A stage is 128
 // of d (or four 16-wide rank-r steps); x slots hold one half's.  TMEM: kNB
 // accumulators of NT columns, then one A stage (128 rows x 128 k, 64 columns)
-// a converter warpgroup.  Up to 128 tokens conversion is most of the work (it
-// does not depend on the tokens): four converter warpgroups; 256 tokens need
-// the registers for 128 accumulators a promotion thread.
+// a converter warpgroup.  Up to 128 tokens a stage's MMAs are short and its
+// conversion is not (it does not depend on the tokens): four converter
+// warpgroups; 256 tokens need the registers for 128 accumulators a promotion
+// thread.
 template <int TM>
 struct PfGeom {
   static constexpr int NT = TM == 64 ? 64 : 128;
@@ -121,7 +125,7 @@ struct PrefillParams {
   int M, num_vt, num_mt, d_pad, G_pad, g, nls, nls_core;
   int nt;  // tokens of an MMA and of an x box, a multiple of 16 up to the instance's NT
   int G_pad2;
-  int blk_log2;  // log2 of a residual block's 16-wide steps (g / 16; SC4: kSc4BlockSteps)
+  int blk_log2;  // log2 of a residual block's 16-wide steps (g / 16; SC4: kSc4BlockLog2)
   void *out;
   int out_fp32;
   const int32_t *targets;  // global vocabulary rows
@@ -824,85 +828,85 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
       if (!mbar_wait_warp(&c_full[cr.s], cr.ph, p.wait_budget, abort_flag, p.err)) goto done;
       const uint8_t *slot = smem + G::kCodeOff + cr.s * G::kCodeSlot;
       const uint8_t *codes = slot + (cw * 64 + lane) * 16;
-          if (e < KC) {
-            // The warp's codes of the stage first (m-tiles 2 cw and 2 cw + 1 of
-            // two 64-wide halves), then the slot is free; one m-tile's
-            // conversion overlaps the store of the one before.
-            uint4 w[4];
+      if (e < KC) {
+        // The warp's codes of the stage first (m-tiles 2 cw and 2 cw + 1 of
+        // two 64-wide halves), then the slot is free; one m-tile's
+        // conversion overlaps the store of the one before.
+        uint4 w[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) w[i] = *reinterpret_cast<const uint4 *>(codes + (i >> 1) * kChunkBytes + (i & 1) * 512);
-            uint32_t q[kSC4 ? 4 : 1];  // SC4: scale-code bytes of rows lane/4 + 8 i
-            uint32_t q1[kSC4 ? 4 : 1];  // and of the second half where g = 32
-            if constexpr (kSC4) {
-              const uint8_t *sb = slot + G::kScaleOff + cw * 32 + (lane >> 2);
+        for (int i = 0; i < 4; ++i) w[i] = *reinterpret_cast<const uint4 *>(codes + (i >> 1) * kChunkBytes + (i & 1) * 512);
+        uint32_t q[kSC4 ? 4 : 1];  // SC4: scale-code bytes of rows lane/4 + 8 i
+        uint32_t q1[kSC4 ? 4 : 1];  // and of the second half where g = 32
+        if constexpr (kSC4) {
+          const uint8_t *sb = slot + G::kScaleOff + cw * 32 + (lane >> 2);
 #pragma unroll
-              for (int i = 0; i < 4; ++i) q[i] = sb[8 * i];
-              if (lg == 5) {
+          for (int i = 0; i < 4; ++i) q[i] = sb[8 * i];
+          if (lg == 5) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) q1[i] = sb[kTileRows + 8 * i];
-              }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&c_empty[cr.s]);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int hf = i >> 1, h = i & 1;
-              uint32_t ah[16];
-              const uint32_t ws[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
-              Sc4Mult lo, hi;  // SC4: multipliers q + 1 of the half's group (two groups where g = 32)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                uint32_t a[4];
-                if constexpr (kSC4) {
-                  if (j == 0 || (j == 2 && lg == 5)) {
-                    const int sh = 4 * (((e * 128 + hf * 64 + 16 * j) >> lg) & 1);
-                    const bool second = hf == 1 && lg == 5;
-                    lo.set(second ? q1[2 * h] : q[2 * h], sh);
-                    hi.set(second ? q1[2 * h + 1] : q[2 * h + 1], sh);
-                  }
-                  unpack_int4x8_biased(ws[j], a);
-                  a[0] = bf16x2_fma(a[0], lo.m, lo.nb);
-                  a[1] = bf16x2_fma(a[1], hi.m, hi.nb);
-                  a[2] = bf16x2_fma(a[2], lo.m, lo.nb);
-                  a[3] = bf16x2_fma(a[3], hi.m, hi.nb);
-                } else {
-                  unpack_int4x8(ws[j], a);
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) ah[4 * j + k] = a[k];
-              }
-              if (h == 0 && hf < G::kAParts) {
-                if (!mbar_wait_warp(ae + hf, aph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
-                tc_fence_after();
-              }
-              tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16) + 32 * hf, ah);
-            }
-          } else {  // four rank-r steps: the first half's 32 columns
-            const uint8_t *lc = slot + (cw * 64 + lane) * 8;
-            const int n = p.nls - 4 * (e - KC);
-            uint2 w[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-              w[i] = i < 4 || n > 2 ? *reinterpret_cast<const uint2 *>(lc + (i >> 1) * kLrStepBytes + (i & 1) * 256)
-                                    : make_uint2(0x80808080u, 0x80808080u);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&c_empty[cr.s]);
-            // (The last part's release: the others come before it.)
-            if (!mbar_wait_warp(ae + G::kAParts - 1, aph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
-            tc_fence_after();
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              uint32_t ah[16];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                uint32_t a[4];
-                unpack_int8x8(w[2 * j + h].x, w[2 * j + h].y, a);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) ah[4 * j + k] = a[k];
-              }
-              tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16), ah);
-            }
+            for (int i = 0; i < 4; ++i) q1[i] = sb[kTileRows + 8 * i];
           }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&c_empty[cr.s]);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int hf = i >> 1, h = i & 1;
+          uint32_t ah[16];
+          const uint32_t ws[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+          Sc4Mult lo, hi;  // SC4: multipliers q + 1 of the half's group (two groups where g = 32)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t a[4];
+            if constexpr (kSC4) {
+              if (j == 0 || (j == 2 && lg == 5)) {
+                const int sh = 4 * (((e * 128 + hf * 64 + 16 * j) >> lg) & 1);
+                const bool second = hf == 1 && lg == 5;
+                lo.set(second ? q1[2 * h] : q[2 * h], sh);
+                hi.set(second ? q1[2 * h + 1] : q[2 * h + 1], sh);
+              }
+              unpack_int4x8_biased(ws[j], a);
+              a[0] = bf16x2_fma(a[0], lo.m, lo.nb);
+              a[1] = bf16x2_fma(a[1], hi.m, hi.nb);
+              a[2] = bf16x2_fma(a[2], lo.m, lo.nb);
+              a[3] = bf16x2_fma(a[3], hi.m, hi.nb);
+            } else {
+              unpack_int4x8(ws[j], a);
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) ah[4 * j + k] = a[k];
+          }
+          if (h == 0 && hf < G::kAParts) {
+            if (!mbar_wait_warp(ae + hf, aph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
+            tc_fence_after();
+          }
+          tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16) + 32 * hf, ah);
+        }
+      } else {  // four rank-r steps: the first half's 32 columns
+        const uint8_t *lc = slot + (cw * 64 + lane) * 8;
+        const int n = p.nls - 4 * (e - KC);
+        uint2 w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+          w[i] = i < 4 || n > 2 ? *reinterpret_cast<const uint2 *>(lc + (i >> 1) * kLrStepBytes + (i & 1) * 256)
+                                : make_uint2(0x80808080u, 0x80808080u);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&c_empty[cr.s]);
+        // (The last part's release: the others come before it.)
+        if (!mbar_wait_warp(ae + G::kAParts - 1, aph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
+        tc_fence_after();
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          uint32_t ah[16];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            uint32_t a[4];
+            unpack_int8x8(w[2 * j + h].x, w[2 * j + h].y, a);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) ah[4 * j + k] = a[k];
+          }
+          tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16), ah);
+        }
+      }
       asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
       tc_fence_before();
       __syncwarp();

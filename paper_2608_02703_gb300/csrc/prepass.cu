@@ -9,7 +9,8 @@
 // tensor-core kernels can apply the rank-r branches with exact int8 codes of
 // A_c and A_w as the other operand.  Outputs: the decode kernel's B-fragment
 // layout of (hi, lo) per 16-token chunk, and/or the prefill kernel's row-major
-// extended operand T = [hi_core | lo_core | hi_corr | lo_corr].
+// extended operand T: per 16 extended columns their 16 hi parts, then their 16
+// lo parts (t_col).
 //
 // Grid: (32 extended columns, 16 tokens, 256-wide split of d).  In a block,
 // warp w takes the 32-wide slice w of its split (a slice never straddles a
