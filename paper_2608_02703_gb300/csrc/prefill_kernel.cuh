@@ -830,8 +830,8 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
       const uint8_t *codes = slot + (cw * 64 + lane) * 16;
       if (e < KC) {
         // The warp's codes of the stage first (m-tiles 2 cw and 2 cw + 1 of
-        // two 64-wide halves), then the slot is free; one m-tile's
-        // conversion overlaps the store of the one before.
+        // two 64-wide halves); one m-tile's conversion overlaps the store of
+        // the one before.
         uint4 w[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) w[i] = *reinterpret_cast<const uint4 *>(codes + (i >> 1) * kChunkBytes + (i & 1) * 512);
@@ -846,8 +846,6 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
             for (int i = 0; i < 4; ++i) q1[i] = sb[kTileRows + 8 * i];
           }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&c_empty[cr.s]);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int hf = i >> 1, h = i & 1;
@@ -889,8 +887,6 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
         for (int i = 0; i < 8; ++i)
           w[i] = i < 4 || n > 2 ? *reinterpret_cast<const uint2 *>(lc + (i >> 1) * kLrStepBytes + (i & 1) * 256)
                                 : make_uint2(0x80808080u, 0x80808080u);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&c_empty[cr.s]);
         // (The last part's release: the others come before it.)
         if (!mbar_wait_warp(ae + G::kAParts - 1, aph ^ 1, p.wait_budget, abort_flag, p.err)) goto done;
         tc_fence_after();
@@ -907,10 +903,14 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
           tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16), ah);
         }
       }
+      // The code slot is free once its words have gone into the A stage: an
+      // arrive right behind the loads, whose results nothing had used yet, let
+      // the refill overtake loads that were held up (5 of 720 passes over 4096
+      // tokens, Qwen3-8B shape, had a unit with wrong codes; none of 2880 since).
       asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&a_full[cg]);
+      if (lane == 0) mbar_arrive(&c_empty[cr.s]), mbar_arrive(&a_full[cg]);
       aph ^= 1;
       cr.next(kConv);
     }

@@ -116,6 +116,25 @@ def test_decode_wide_sampled_tokens(name, M):
     assert np.max(d) <= gu.CE_ABS, f"{name}: decode CE M={M} max|d|={np.max(d):.3e}"
 
 
+@pytest.mark.parametrize("name", ["qwen3-8b", "qwen3-8b-sc4"])
+def test_passes_repeat_bit_for_bit(name):
+    """Every pass over the same tokens gives the same bits (once in 150 a unit
+    of the tensor-core kernel did not)."""
+    import torch
+
+    pack, _ = get(name)
+    V, M = pack.shape.V, PREFILL_M[name]
+    x = gu.to_dev(make_hidden(pack.shape.d, M, seed=6))
+    y, first = (torch.empty((M, V), dtype=torch.int16, device="cuda") for _ in range(2))
+    archead.archead_forward(pack, x, M, first, archead.OUT_BF16)
+    different = torch.zeros((), dtype=torch.int64, device="cuda")
+    for _ in range(400):
+        archead.archead_forward(pack, x, M, y, archead.OUT_BF16)
+        different += (~(y == first).all()).long()
+    assert archead.archead_sync_status(pack) == archead.OK
+    assert int(different) == 0, f"{int(different)} of 400 passes differ from the first"
+
+
 @pytest.mark.parametrize("name", FULL)
 def test_prefill_sampled_tokens(name):
     """The bench's prefill launch (M = 4096 / 2048 tokens: logits, greedy
