@@ -90,8 +90,9 @@ def test_greedy_full_vocabulary(name):
 @pytest.mark.parametrize("M", [27, 64])
 def test_decode_wide_sampled_tokens(name, M):
     """One launch of the 32- resp. 64-token decode instance (every n-tile of
-    the launch, the ragged one included) over the whole vocabulary: logits,
-    greedy output and fused CE on one token of each 8-token n-tile."""
+    the launch, the ragged one included) and the kernel that AUTO takes, over
+    the whole vocabulary: logits, greedy output and fused CE on one token of
+    each 8-token n-tile."""
     import torch
 
     pack, head = get(name)
@@ -100,39 +101,46 @@ def test_decode_wide_sampled_tokens(name, M):
     t = make_targets(shape.V, M, seed=4)
     idx = np.unique(np.minimum(np.arange(0, M + 7, 8) + (np.arange(0, M + 7, 8) // 8) % 8, M - 1))
     ref = oracle.logits(head, shape, x[idx])
-    y = torch.full((M, shape.V), float("nan"), dtype=torch.float32, device="cuda")
-    archead.archead_forward(pack, gu.to_dev(x), M, y, archead.OUT_FP32)
-    assert archead.archead_sync_status(pack) == archead.OK
-    got = _rows(y, torch.from_numpy(idx).cuda())
-    gu.check_logits(got, ref, where=f"{name} decode M={M} sampled")
-    gu.check_argmax(got, ref, where=f"{name} decode M={M} sampled")
-    del y
-    gi, gv = gu.forward_argmax(pack, x)
-    gu.check_greedy(gi[idx], gv[idx], ref, where=f"{name} decode greedy M={M} sampled")
-    ce, st = gu.forward_ce(pack, x, t)
-    assert st == archead.OK
     ref_ce = oracle.cross_entropy(head, shape, x[idx], t[idx])
-    d = np.abs(ce[idx] - ref_ce["ce"])
-    assert np.max(d) <= gu.CE_ABS, f"{name}: decode CE M={M} max|d|={np.max(d):.3e}"
+    for path in (archead.PATH_DECODE, archead.PATH_AUTO):
+        y = torch.full((M, shape.V), float("nan"), dtype=torch.float32, device="cuda")
+        archead.archead_forward_path(pack, gu.to_dev(x), M, y, archead.OUT_FP32, path)
+        assert archead.archead_sync_status(pack) == archead.OK
+        got = _rows(y, torch.from_numpy(idx).cuda())
+        gu.check_logits(got, ref, where=f"{name} path={path} M={M} sampled")
+        gu.check_argmax(got, ref, where=f"{name} path={path} M={M} sampled")
+        del y
+        gi, gv = gu.forward_argmax(pack, x, path)
+        gu.check_greedy(gi[idx], gv[idx], ref, where=f"{name} path={path} greedy M={M} sampled")
+        ce, st = gu.forward_ce(pack, x, t, path)
+        assert st == archead.OK
+        d = np.abs(ce[idx] - ref_ce["ce"])
+        assert np.max(d) <= gu.CE_ABS, f"{name}: path={path} CE M={M} max|d|={np.max(d):.3e}"
 
 
 @pytest.mark.parametrize("name", ["qwen3-8b", "qwen3-8b-sc4"])
-def test_passes_repeat_bit_for_bit(name):
-    """Every pass over the same tokens gives the same bits (once in 150 a unit
-    of the tensor-core kernel did not)."""
+@pytest.mark.parametrize("M,path,passes", [
+    (4096, archead.PATH_PREFILL, 400), (100, archead.PATH_PREFILL, 1000), (24, archead.PATH_PREFILL, 1000),
+    (1, archead.PATH_DECODE, 2000), (8, archead.PATH_DECODE, 2000), (16, archead.PATH_DECODE, 1000),
+    (64, archead.PATH_DECODE, 500),
+])
+def test_passes_repeat_bit_for_bit(name, M, path, passes):
+    """Every pass over the same tokens gives the same bits.  (Both kernels copy
+    stages to registers and hand the slot back; loads that slipped behind the
+    hand-back once gave a unit of 4096 tokens wrong codes, in a pass of 150.)"""
     import torch
 
     pack, _ = get(name)
-    V, M = pack.shape.V, PREFILL_M[name]
+    V = pack.shape.V
     x = gu.to_dev(make_hidden(pack.shape.d, M, seed=6))
     y, first = (torch.empty((M, V), dtype=torch.int16, device="cuda") for _ in range(2))
-    archead.archead_forward(pack, x, M, first, archead.OUT_BF16)
+    archead.archead_forward_path(pack, x, M, first, archead.OUT_BF16, path)
     different = torch.zeros((), dtype=torch.int64, device="cuda")
-    for _ in range(400):
-        archead.archead_forward(pack, x, M, y, archead.OUT_BF16)
+    for _ in range(passes):
+        archead.archead_forward_path(pack, x, M, y, archead.OUT_BF16, path)
         different += (~(y == first).all()).long()
     assert archead.archead_sync_status(pack) == archead.OK
-    assert int(different) == 0, f"{int(different)} of 400 passes differ from the first"
+    assert int(different) == 0, f"{int(different)} of {passes} passes differ from the first"
 
 
 @pytest.mark.parametrize("name", FULL)
