@@ -903,9 +903,9 @@ __global__ void __launch_bounds__(PfGeom<TM>::kThreads, 1) prefill_kernel(const 
           tmem_st_frag4(acol + ((uint32_t)(16 * h) << 16), ah);
         }
       }
-      // The code slot is free once its words have gone into the A stage: an
-      // arrive right behind the loads, whose results nothing had used yet, let
-      // the refill overtake loads that were held up (5 of 720 passes over 4096
+      // The code slot is free once its words have gone into the A stage.  An
+      // arrive right behind the loads had some of them moved behind it by the
+      // compiler, where the refill could meet them (5 of 720 passes over 4096
       // tokens, Qwen3-8B shape, had a unit with wrong codes; none of 2880 since).
       asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
       tc_fence_before();
